@@ -97,14 +97,6 @@ __device__ __forceinline__ void tmem_ld64(uint32_t taddr, float *v) {
     for (int i = 0; i < 64; ++i) v[i] = __uint_as_float(r[i]);
 }
 
-__global__ void max_kernel(const float *v, int64_t n, float *out) {
-    float m = 0.f;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        m = fmaxf(m, v[i]);
-    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-    if ((threadIdx.x & 31) == 0) atomicMax((int *)out, __float_as_int(m));   // m >= 0
-}
-
 // Exact re-rank and certificate, one warp per query.
 __global__ void rerank_certify_kernel(const float *X, const float *Q, int d, int metric, int64_t nq,
                                       int k, int K1, const float *cand_d, const int32_t *cand_i,
@@ -717,42 +709,86 @@ __global__ void __launch_bounds__(kThreads2, 1) tc_knn2_kernel(Tc2Args a) {
     }
 }
 
-// One thread per (row, 8 dimensions) of the padded matrix: FP32 -> BF16 hi
-// and lo parts, written into the tiled, swizzled block layout. Row `i` of the
-// output is input row order[i] (or i), rows past `rows` are zero.
-__global__ void tile_split_kernel(const float *X, int64_t rows, int d, int nk, const int32_t *order,
-                                  int64_t rows_pad, unsigned char *out) {
-    const int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (idx >= rows_pad * nk * 8) return;
-    const int64_t row = idx / (nk * 8);
-    const int g = (int)(idx % (nk * 8));
-    const int kc = g >> 3, c = g & 7;
+// FP32 rows -> BF16 hi and lo parts in the tiled, swizzled block layout, and
+// the rows' squared norms (and norms, and their maximum), in one pass. LR
+// lanes share a row: lane `sub` takes its 8-dimension groups sub, sub + LR,
+// ..., two 16-byte loads each, stores both 16-byte parts and adds up the
+// squares, which are summed over the LR lanes by shuffles. Row `i` of the
+// output is input row order[i] (or i), rows past `rows` are zero; norms are
+// written at the input row, and nothing for padding rows.
+// Memory bound: 4 d bytes read and 4 * 64 nk written per row. LR is the largest
+// power of two up to 32 that divides the row's 8 nk groups, so that no lane is
+// idle and a warp's loads are whole 128-byte lines. Norms apart (one thread
+// per row, uncoalesced) took 418 us at 1M x 128 and 576 us at 200,003 x 768,
+// beside 143 and 172 us for the split; one pass takes 153 us (6.7 TB/s) and 172 us.
+template <int LR>
+__global__ void __launch_bounds__(256) split_norm_kernel(const float *__restrict__ X, int64_t rows, int d, int nk,
+                                                         const int32_t *__restrict__ order, int64_t rows_pad,
+                                                         unsigned char *__restrict__ out, float *norm,
+                                                         float *rownorm, float *max_rownorm) {
+    const int sub = threadIdx.x % LR;
+    const int64_t row = blockIdx.x * (int64_t)(256 / LR) + threadIdx.x / LR;
     const int64_t src = row < rows ? (order ? (int64_t)order[row] : row) : -1;
-    __align__(16) __nv_bfloat16 h[8];
-    __align__(16) __nv_bfloat16 lo[8];
-#pragma unroll
-    for (int e = 0; e < 8; ++e) {
-        const int k = kc * TK + c * 8 + e;
-        const float v = (src >= 0 && k < d) ? X[src * d + k] : 0.f;
-        h[e] = __float2bfloat16_rn(v);
-        lo[e] = __float2bfloat16_rn(v - __bfloat162float(h[e]));
-    }
     const int64_t tile = row >> 7;
     const int t = (int)(row & 127);
-    unsigned char *blk = out + (tile * nk + kc) * (int64_t)STAGE;
-    const uint32_t off = t * 128 + ((c ^ (t & 7)) << 4);
-    *(uint4 *)(blk + off) = *(const uint4 *)h;
-    *(uint4 *)(blk + CHUNK + off) = *(const uint4 *)lo;
+    float s = 0.f;
+    if (row < rows_pad) {
+        for (int g = sub; g < nk * 8; g += LR) {
+            const int k = g * 8;
+            float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b = a;
+            if (src >= 0 && k < d) {   // d % 4 == 0 and 16-byte aligned rows
+                const float4 *x4 = reinterpret_cast<const float4 *>(X + src * d + k);
+                a = __ldg(x4);
+                if (k + 4 < d) b = __ldg(x4 + 1);
+            }
+            const float v[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+            __align__(16) __nv_bfloat16 h[8];
+            __align__(16) __nv_bfloat16 lo[8];
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                h[e] = __float2bfloat16_rn(v[e]);
+                lo[e] = __float2bfloat16_rn(v[e] - __bfloat162float(h[e]));
+                s = fmaf(v[e], v[e], s);
+            }
+            unsigned char *blk = out + (tile * nk + (g >> 3)) * (int64_t)STAGE;
+            const uint32_t off = t * 128 + (((g & 7) ^ (t & 7)) << 4);
+            *(uint4 *)(blk + off) = *(const uint4 *)h;
+            *(uint4 *)(blk + CHUNK + off) = *(const uint4 *)lo;
+        }
+    }
+#pragma unroll
+    for (int o = LR >> 1; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    const float rn = sqrtf(s);
+    if (sub == 0 && src >= 0) {
+        norm[src] = s;
+        if (rownorm) rownorm[src] = rn;
+    }
+    if (max_rownorm) {
+        float m = fmaxf(src >= 0 ? rn : 0.f, 0.f);   // a NaN row does not count
+#pragma unroll
+        for (int o = 16; o >= LR && o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+        __shared__ float wm[8];
+        if ((threadIdx.x & 31) == 0) wm[threadIdx.x >> 5] = m;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            for (int w = 1; w < 8; ++w) m = fmaxf(m, wm[w]);
+            atomicMax((int *)max_rownorm, __float_as_int(m));   // m >= 0
+        }
+    }
 }
 
-__global__ void norms_kernel(const float *X, int64_t rows, int d, float *norm, float *rownorm) {
-    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= rows) return;
-    const float *x = X + i * d;
-    float s = 0.f;
-    for (int j = 0; j < d; ++j) s = fmaf(x[j], x[j], s);
-    norm[i] = s;
-    rownorm[i] = sqrtf(s);
+// Launches split_norm_kernel with the lanes per row of nk 64-wide chunks.
+cudaError_t split_norm(const float *X, int64_t rows, int d, int nk, const int32_t *order, int64_t rows_pad,
+                       unsigned char *out, float *norm, float *rownorm, float *max_rownorm, cudaStream_t stream) {
+    const int lr = nk % 4 == 0 ? 32 : (nk % 2 == 0 ? 16 : 8);
+    const int grid = ceil_div_i(rows_pad, 256 / lr);
+    if (lr == 32)
+        split_norm_kernel<32><<<grid, 256, 0, stream>>>(X, rows, d, nk, order, rows_pad, out, norm, rownorm, max_rownorm);
+    else if (lr == 16)
+        split_norm_kernel<16><<<grid, 256, 0, stream>>>(X, rows, d, nk, order, rows_pad, out, norm, rownorm, max_rownorm);
+    else
+        split_norm_kernel<8><<<grid, 256, 0, stream>>>(X, rows, d, nk, order, rows_pad, out, norm, rownorm, max_rownorm);
+    return cudaGetLastError();
 }
 
 // Merge the per-item top-K1 lists of each valid query (one warp per sorted
@@ -862,11 +898,11 @@ static esg_status bf2_smem(int32_t d, int K1, int max_smem, int *S, size_t *smem
     return ESG_OK;
 }
 
-// The point side, prepared once per call: tiled BF16 splits, squared norms,
-// row norms and their maximum.
+// The point side, prepared once per call: tiled BF16 splits, squared norms
+// and the largest row norm.
 struct PreparedX {
     const unsigned char *xs;
-    const float *xnorm, *xrow, *xmax;
+    const float *xnorm, *xmax;
 };
 
 __global__ void gather_subset_kernel(const float *Q, const int64_t *l, const int64_t *r, int d,
@@ -1284,11 +1320,8 @@ static esg_status bf2_queries(const PreparedX &X, const float *base, int64_t n, 
     if (ce == cudaSuccess)
         ce = cudaMemcpyAsync(d_cta, cta_first.data(), sizeof(int32_t) * (G + 1), cudaMemcpyHostToDevice, stream);
     if (ce == cudaSuccess) {
-        norms_kernel<<<ceil_div_i(nq, 256), 256, 0, stream>>>(queries, nq, d, qnorm, qrow);
         if (nqt > 0)
-            tile_split_kernel<<<ceil_div_i(nqt * TM * nk * 8, 256), 256, 0, stream>>>(queries, nv, d, nk, d_order,
-                                                                                     nqt * TM, qs);
-        ce = cudaGetLastError();
+            ce = split_norm(queries, nv, d, nk, d_order, nqt * TM, qs, qnorm, qrow, nullptr, stream);
     }
     if (ce == cudaSuccess) ce = cudaFuncSetAttribute(tc_knn2_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (ce == cudaSuccess && n_items > 0) {
@@ -1371,21 +1404,17 @@ static esg_status bruteforce_tc_v2(const float *base, int64_t n, int32_t d, int 
     ESG_CUDA_TRY(cudaMemcpyAsync(hr.data(), r, sizeof(int64_t) * nq, cudaMemcpyDeviceToHost, stream));
     ESG_CUDA_TRY(cudaStreamSynchronize(stream));
     auto al = [](size_t x) { return (x + 255) & ~(size_t)255; };
-    const size_t bytes = al((size_t)xt * nk * STAGE) + 2 * al(sizeof(float) * n) + al(sizeof(float) * 4);
+    const size_t bytes = al((size_t)xt * nk * STAGE) + al(sizeof(float) * n) + al(sizeof(float) * 4);
     unsigned char *scratch = nullptr;
     ESG_CUDA_TRY(esg_malloc_async((void **)&scratch, bytes, stream));
     unsigned char *p = scratch;
     unsigned char *xs = p; p += al((size_t)xt * nk * STAGE);
     float *xnorm = (float *)p; p += al(sizeof(float) * n);
-    float *xrow = (float *)p; p += al(sizeof(float) * n);
     float *xmax = (float *)p;
     esg_status st = ESG_OK;
     cudaError_t ce = cudaMemsetAsync(xmax, 0, sizeof(float) * 4, stream);
     if (ce == cudaSuccess) {
-        norms_kernel<<<ceil_div_i(n, 256), 256, 0, stream>>>(base, n, d, xnorm, xrow);
-        max_kernel<<<152, 256, 0, stream>>>(xrow, n, xmax);
-        tile_split_kernel<<<ceil_div_i(xt * TN * nk * 8, 256), 256, 0, stream>>>(base, n, d, nk, nullptr, xt * TN, xs);
-        ce = cudaGetLastError();
+        ce = split_norm(base, n, d, nk, nullptr, xt * TN, xs, xnorm, nullptr, xmax, stream);
     }
     if (ce != cudaSuccess) { esg_set_error(cudaGetErrorString(ce)); st = ESG_ERR_CUDA; }
     const double t1 = bf_stats() ? bf_host_ms() : 0.0;
@@ -1394,7 +1423,7 @@ static esg_status bruteforce_tc_v2(const float *base, int64_t n, int32_t d, int 
     if (bf_stats()) fprintf(stderr, "tensor-core brute force, host ms: ranges + point prep queued %.3f, plan %.3f\n",
                             t1 - t0, bf_host_ms() - t1);
     if (st == ESG_OK) {
-        const PreparedX X{xs, xnorm, xrow, xmax};
+        const PreparedX X{xs, xnorm, xmax};
         st = bf2_queries(X, base, n, d, metric, queries, nq, l, r, k, K1, out_ids, out_dist, out_count, stream, &P);
     }
     cudaFreeAsync(scratch, stream);
