@@ -517,7 +517,9 @@ esg_status esg_bruteforce_filtered_knn(const float *base, int64_t n, int32_t d, 
  * contiguous shares (fewer when there are fewer covered tiles) of about equal
  * estimated cost: tiles + 6.25 (2 / ceil(d / 64))^2 per (query, work item)
  * pair in which the query covers one of the item's tiles; a share is split
- * into work items at query-tile boundaries.
+ * into work items at query-tile boundaries. A search plans the same order and
+ * tiles; its cuts weigh a query whose range begins inside a work item more than
+ * one whose list starts with it, and narrow ranges by their tiles.
  *  n, d       points and dimension of the search (d sets the cost weight);
  *  l, r       host [nq] int64 inclusive ranges;
  *  ctas       CTAs to plan for (the kernel uses one per SM);

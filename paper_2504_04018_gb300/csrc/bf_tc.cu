@@ -10,12 +10,12 @@
 // thread, and eight epilogue warps that keep the K1 best approximate
 // distances per query.
 //
-// A second kernel recomputes exact FP32 distances (direct form) of those
-// candidates, sorts them, and certifies the result: with delta_q a bound on
-// |approximate - exact| for every point of the range, the top k is proven
-// when the exact k-th distance is below (K1-th approximate distance -
-// delta_q). Queries without a certificate run again with a longer list, then
-// through the exact SIMT brute force.
+// A second kernel merges a query's lists, recomputes exact FP32 distances
+// (direct form) of the K1 best candidates, sorts them, and certifies the
+// result: with delta_q a bound on |approximate - exact| for every point of the
+// range, the top k is proven when the exact k-th distance is below (K1-th
+// approximate distance - delta_q). Queries without a certificate run again
+// with a longer list, then through the exact SIMT brute force.
 #include "esg_internal.cuh"
 
 #include <algorithm>
@@ -23,6 +23,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
+#include <type_traits>
 #include <vector>
 
 esg_status esg_bruteforce_redo(const float *base, int64_t n, int32_t d, int metric, const float *queries,
@@ -66,99 +67,136 @@ __device__ __forceinline__ void mma_bf16(uint32_t tmem_d, uint64_t a, uint64_t b
         :: "r"(tmem_d), "l"(a), "l"(b), "r"(kIdesc), "r"(acc));
 }
 
+// The same with the A operand in tensor memory: row i in lane i, 16 BF16 of K
+// packed in pairs in 8 columns from tmem_a on.
+__device__ __forceinline__ void mma_bf16_ta(uint32_t tmem_d, uint32_t tmem_a, uint64_t b, uint32_t acc) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}\n"
+        :: "r"(tmem_d), "r"(tmem_a), "l"(b), "r"(kIdesc), "r"(acc));
+}
+
 __device__ __forceinline__ void mma_commit(uint32_t mbar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
                  :: "r"(mbar) : "memory");
 }
 
-// 64 consecutive accumulator columns of the warp's 32 TMEM lanes (one
+// 32 consecutive accumulator columns of the warp's 32 TMEM lanes (one
 // register each), waiting for the load inside the same asm statement so that
 // no use of the registers can be scheduled before the wait.
-__device__ __forceinline__ void tmem_ld64(uint32_t taddr, float *v) {
-    uint32_t r[64];
+__device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
+    uint32_t r[32];
     asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x64.b32 "
+        "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
         "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,"
-        "%25,%26,%27,%28,%29,%30,%31,%32,%33,%34,%35,%36,%37,%38,%39,%40,%41,%42,%43,%44,%45,%46,"
-        "%47,%48,%49,%50,%51,%52,%53,%54,%55,%56,%57,%58,%59,%60,%61,%62,%63}, [%64];\n\t"
+        "%25,%26,%27,%28,%29,%30,%31}, [%32];\n\t"
         "tcgen05.wait::ld.sync.aligned;"
         : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
           "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]),
           "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]),
           "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]),
-          "=r"(r[29]), "=r"(r[30]), "=r"(r[31]), "=r"(r[32]), "=r"(r[33]), "=r"(r[34]), "=r"(r[35]),
-          "=r"(r[36]), "=r"(r[37]), "=r"(r[38]), "=r"(r[39]), "=r"(r[40]), "=r"(r[41]), "=r"(r[42]),
-          "=r"(r[43]), "=r"(r[44]), "=r"(r[45]), "=r"(r[46]), "=r"(r[47]), "=r"(r[48]), "=r"(r[49]),
-          "=r"(r[50]), "=r"(r[51]), "=r"(r[52]), "=r"(r[53]), "=r"(r[54]), "=r"(r[55]), "=r"(r[56]),
-          "=r"(r[57]), "=r"(r[58]), "=r"(r[59]), "=r"(r[60]), "=r"(r[61]), "=r"(r[62]), "=r"(r[63])
+          "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
         : "r"(taddr)
         : "memory");
 #pragma unroll
-    for (int i = 0; i < 64; ++i) v[i] = __uint_as_float(r[i]);
+    for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
 }
 
-// Exact re-rank and certificate, one warp per query.
-__global__ void rerank_certify_kernel(const float *X, const float *Q, int d, int metric, int64_t nq,
-                                      int k, int K1, const float *cand_d, const int32_t *cand_i,
-                                      const int32_t *cand_n, const float *qrownorm, const float *xmax,
-                                      int64_t *out_ids, float *out_dist,
-                                      int32_t *out_count, int32_t *redo) {
-    __shared__ Cand buf[4][128];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int64_t q = blockIdx.x * (int64_t)(blockDim.x >> 5) + w;
-    if (q >= nq) return;
-    Cand *b = buf[w];
-    const int m = cand_n[q];
-    if (m < 0) {  // invalid range
-        for (int j = lane; j < k; j += 32) { out_ids[q * k + j] = -1; out_dist[q * k + j] = INFINITY; }
-        if (lane == 0) { out_count[q] = 0; redo[q] = 0; }
-        return;
-    }
-    const float *qq = Q + q * (int64_t)d;
-    for (int e = 0; e < m; ++e) {
-        const int32_t row = cand_i[q * K1 + e];
-        const float *x = X + (int64_t)row * d;
-        float acc = 0.f;
-        for (int j = lane; j < d; j += 32) {
-            if (metric == ESG_L2SQ) { const float t = qq[j] - x[j]; acc = fmaf(t, t, acc); }
-            else acc = fmaf(qq[j], x[j], acc);
+// 32 words per lane into 32 consecutive columns of the warp's 32 TMEM lanes.
+__device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint4 (&w)[8]) {
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], "
+        "{%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,"
+        "%28,%29,%30,%31,%32};"
+        :: "r"(taddr), "r"(w[0].x), "r"(w[0].y), "r"(w[0].z), "r"(w[0].w), "r"(w[1].x), "r"(w[1].y), "r"(w[1].z),
+           "r"(w[1].w), "r"(w[2].x), "r"(w[2].y), "r"(w[2].z), "r"(w[2].w), "r"(w[3].x), "r"(w[3].y), "r"(w[3].z),
+           "r"(w[3].w), "r"(w[4].x), "r"(w[4].y), "r"(w[4].z), "r"(w[4].w), "r"(w[5].x), "r"(w[5].y), "r"(w[5].z),
+           "r"(w[5].w), "r"(w[6].x), "r"(w[6].y), "r"(w[6].z), "r"(w[6].w), "r"(w[7].x), "r"(w[7].y), "r"(w[7].z),
+           "r"(w[7].w)
+        : "memory");
+}
+
+// ---------------------------------------------------------- candidate lists
+// A list entry is one 64-bit key: the distance's bits mapped to an unsigned
+// that orders like the float, above the point's row, so that comparing keys
+// orders by (distance, row). Lists and batches are held across a warp's lanes
+// (element e = lane + 32 h in register h) and padded with kPad.
+typedef unsigned long long Key;
+constexpr Key kPad = ~0ull;
+
+__device__ __forceinline__ Key make_key(float d, uint32_t row) {
+    const uint32_t b = __float_as_uint(d);
+    return ((Key)(b ^ ((uint32_t)((int32_t)b >> 31) | 0x80000000u)) << 32) | row;
+}
+__device__ __forceinline__ float key_dist(Key k) {
+    const uint32_t b = (uint32_t)(k >> 32);
+    return __uint_as_float((b & 0x80000000u) ? (b ^ 0x80000000u) : ~b);
+}
+__device__ __forceinline__ Key key_min(Key a, Key b) { return a < b ? a : b; }
+__device__ __forceinline__ Key key_max(Key a, Key b) { return a < b ? b : a; }
+
+// A bitonic sequence of 32 NL keys sorted ascending.
+template <int NL>
+__device__ __forceinline__ void bitonic_asc(Key (&L)[NL], int lane) {
+#pragma unroll
+    for (int j = 16 * NL; j >= 32; j >>= 1)
+#pragma unroll
+        for (int h = 0; h < NL; ++h)
+            if ((h & (j >> 5)) == 0) {
+                const Key a = L[h], b = L[h | (j >> 5)];
+                L[h] = key_min(a, b);
+                L[h | (j >> 5)] = key_max(a, b);
+            }
+#pragma unroll
+    for (int j = 16; j > 0; j >>= 1)
+#pragma unroll
+        for (int h = 0; h < NL; ++h) {
+            const Key o = __shfl_xor_sync(0xffffffffu, L[h], j);
+            L[h] = (lane & j) ? key_max(L[h], o) : key_min(L[h], o);
         }
-        acc = warp_sum_group(acc, 32);
-        if (lane == 0) b[e] = Cand{metric == ESG_L2SQ ? acc : -acc, (uint32_t)row};
-    }
-    __syncwarp();
-    const int P = 128;
-    for (int j = m + lane; j < P; j += 32) b[j] = Cand{INFINITY, ESG_NONE};
-    __syncwarp();
-    warp_sort_pow2(b, P);
-    const int c = min(k, m);
-    bool certified = c > 0;
-    if (m == K1) {   // the list is full: points may have been left out
-        // |approximate - exact| for any point of the range (unit roundoff of
-        // BF16 2^-8, of FP32 2^-24): the split residuals and the dropped
-        // lo*lo product stay below 3.1 * 2^-16 |q_i||x_i| per term, the FP32
-        // accumulation of 3d products below 6d * 2^-24 (twice the rounding
-        // bound, for truncating adders); the squared distance doubles the dot
-        // product error and adds the rounding of the norms and the final sum.
-        const double qn = qrownorm[q], xm = xmax[0];
-        const double dot_err = (3.1 * 0x1p-16 + 6.0 * d * 0x1p-24) * qn * xm;
-        const double delta = metric == ESG_L2SQ ? 2.0 * dot_err + (d + 4.0) * 0x1p-24 * (qn * qn + xm * xm)
-                                                : dot_err;
-        const double bound = (double)cand_d[q * K1 + K1 - 1] - delta;
-        // the re-ranked FP32 distance itself is within d * 2^-23 relative
-        const double dk = (double)b[c - 1].d;
-        certified = dk + fabs(dk) * d * 0x1p-23 < bound;
-    }
-    for (int j = lane; j < k; j += 32) {
-        out_ids[q * k + j] = j < c ? (int64_t)b[j].id : -1;
-        out_dist[q * k + j] = j < c ? b[j].d : INFINITY;
-    }
-    if (lane == 0) { out_count[q] = c; redo[q] = certified ? 0 : 1; }
 }
 
+// The 32 NL smallest keys of two ascending lists, ascending, into A. Element
+// e of A meets element 32 NL - 1 - e of B.
+template <int NL>
+__device__ __forceinline__ void merge_lists(Key (&A)[NL], const Key (&B)[NL], int lane) {
+    Key rev[NL];
+#pragma unroll
+    for (int h = 0; h < NL; ++h) rev[h] = __shfl_sync(0xffffffffu, B[NL - 1 - h], 31 - lane);
+#pragma unroll
+    for (int h = 0; h < NL; ++h) A[h] = key_min(A[h], rev[h]);
+    bitonic_asc<NL>(A, lane);
+}
+
+// Full ascending sort of 32 NL keys.
+template <int NL>
+__device__ __forceinline__ void sort_asc(Key (&L)[NL], int lane) {
+#pragma unroll
+    for (int kk = 2; kk <= 32 * NL; kk <<= 1)
+#pragma unroll
+        for (int j = kk >> 1; j > 0; j >>= 1) {
+            if (j >= 32) {
+#pragma unroll
+                for (int h = 0; h < NL; ++h)
+                    if ((h & (j >> 5)) == 0) {
+                        const Key a = L[h], b = L[h | (j >> 5)];
+                        const bool up = ((32 * h) & kk) == 0;
+                        L[h] = up ? key_min(a, b) : key_max(a, b);
+                        L[h | (j >> 5)] = up ? key_max(a, b) : key_min(a, b);
+                    }
+            } else {
+#pragma unroll
+                for (int h = 0; h < NL; ++h) {
+                    const Key o = __shfl_xor_sync(0xffffffffu, L[h], j);
+                    const bool keep_min = (((lane + 32 * h) & kk) == 0) == ((lane & j) == 0);
+                    L[h] = keep_min ? key_min(L[h], o) : key_max(L[h], o);
+                }
+            }
+        }
+}
 
 // ------------------------------------------------------------------------
-// Pipelined version. The operands are pre-tiled in global memory in exactly
+// Pipelined kernel. The operands are pre-tiled in global memory in exactly
 // the shared-memory layout the MMA descriptors name (one 32 KB block per
 // 128 rows x 64 dimensions: BF16 hi part, then lo part, 128-byte swizzle,
 // zero padding past the last row and dimension), so every stage is one bulk
@@ -167,29 +205,63 @@ __global__ void rerank_certify_kernel(const float *X, const float *Q, int d, int
 // that its queries' ranges cover; the CTAs (one per SM) run contiguous
 // shares of that sequence of equal estimated cost, cut into work items at
 // query-tile boundaries. Each CTA is warp-specialised:
-//   warp 0      bulk copies: the item's query tile (resident), then a ring of
-//               S point-tile stages;
-//   warp 1      one thread issues the MMAs into one of two TMEM accumulators
-//               (128 columns each) and commits them to mbarriers;
-//   warps 2..9  epilogue: each reads half a row (64 columns) of the finished
-//               accumulator into registers and releases it; the tile is then
-//               passed through shared memory half by half so that one warp
-//               handles one query row at a time: range mask, distance, a
-//               ballot against the row's current K1-th distance, and, for the
-//               rare candidates that pass, an insertion into the row's sorted
-//               list held across the warp's lanes. A CTA runs a contiguous
-//               share of the items, so a row's list carries over between its
-//               items of the same query tile; the lists go to global memory
-//               and a merge kernel combines them per query.
+//   warp 0      bulk copies: a ring of S point-tile stages (d <= 256), or of
+//               stages with a query and a point chunk (streamed, larger d);
+//   warps 1, 2  one thread each issues the MMAs of alternate tiles (warp 1 all
+//               of them where a tile's stages are over half of the ring) into
+//               a ring of 2 to 4 TMEM accumulators (128 columns each) and
+//               commits them to mbarriers;
+//   warps 3..10 epilogue, two groups of four warps (one per TMEM lane
+//               quarter) that take alternate tiles. A thread owns one query
+//               row: it reads the row's 128 columns 8 or 16 at a time, compares
+//               each distance with the row's threshold and appends the few
+//               that pass to the row's pending slots in shared memory. When a
+//               row's slots run low its warp sorts them in registers and
+//               merges them into the row's sorted list in global memory (32
+//               NL keys across the lanes, the loads overlapped with the
+//               sort), which lowers the threshold. At d <= 256 group 0 also
+//               puts the item's query tile into tensor memory (64 columns per
+//               64 dimensions): the MMAs then read only the point operand from
+//               shared memory, which at N = 128 otherwise limits them, and
+//               all of it holds point stages.
+// The eight warps share nothing but the thresholds: each (row, group) has its
+// own list, so no warp waits for another one, and a row uses the other
+// group's published distances, tagged with the work item: no point above t is
+// among the K1 best when one list has K1 points up to t, or both have half as
+// many.
+// A row of a narrow range instead writes all its distances to global memory
+// (a dense row, see kDenseWidth); the finish kernel selects from them.
+// What bounds it: at 1M x 128 (10k queries, k = 10) a point tile is 24 MMAs,
+// 0.74 us, and the CTAs take 1.1 to 1.2 us per tile: an accumulator is held for
+// the MMAs and then for the group's reading, three of them are in turn, and
+// everything that passes the shared-memory crossbar (norms, shuffles, pending
+// slots) competes with the MMAs' operand reads. 4.67 -> 2.0 ms for the kernel,
+// 1.52 -> 1.07 ms at 200,003 x 768 (2k queries), 256 -> 18 us for 61 queries over
+// 99,991 x 100. Tried on the way: one issuer (a thread's waits and commits cost
+// as much as a stage's MMAs), lists sorted by shuffle networks of 4 or 8 rows
+// (1,100 to 1,900 cycles a row under the crossbar's load; all 32 rows of a warp
+// insert into register lists in 4,000 to 5,000), the query tile in shared memory.
 // Every wait is bounded (2 s of global time); a wait that runs out sets the
 // error flag and all roles leave their loops.
 
 constexpr int STAGE = 2 * CHUNK;          // hi + lo of a 128 x 64 block
 constexpr int kEpiWarps = 8;
-constexpr int kThreads2 = 64 + 32 * kEpiWarps;
-constexpr int kMaxK1v2 = 64;
-constexpr int kTS = 65;                   // row stride of the transposed half tile
+constexpr int kMmaWarps = 2;
+constexpr int kThreads2 = 32 + 32 * kMmaWarps + 32 * kEpiWarps;
+constexpr int kMaxK1v2 = 64;              // longest list
 constexpr int kMaxStages = 6;
+constexpr int kTmem = 512;                // TMEM columns: all, one CTA per SM
+constexpr int kMaxResident = 4;           // 64-wide chunks of a query tile that fit beside two accumulators
+// Columns between two checks of the pending slots, slots per row (a check's
+// columns must fit, at most 32: one per lane of the sort), and how many of
+// them make a row worth merging along with one that has to be. 20 slots leave
+// room for four stages and the lists at d = 128, K1 = 22; 12 for three streamed
+// stages.
+constexpr int kCols = 8;
+template <bool STREAM> struct Epi {
+    static constexpr int kPend = STREAM ? 12 : 20, kFill = STREAM ? 4 : 8;
+};
+constexpr int kPendStride = 33;           // slots of one row 33 entries apart: no bank conflict when read
 // Limit of the waits that let work already issued finish before a CTA exits
 // (bulk copies, MMAs); the pipeline's own waits take Tc2Args::wait_ns.
 constexpr unsigned long long kWaitNs = 2000000000ull;
@@ -203,17 +275,20 @@ struct Tc2Args {
     const float *xnorm, *qnorm;     // squared norms (queries in caller order)
     const int64_t *l, *r;
     const int32_t *qorder;          // sorted position -> caller's query index
+    const int64_t *doff;            // sorted position -> first entry of a dense row, or -1
+    float *dense;                   // distances of the dense rows' ranges, from point l & ~3 on
     const WorkItem *items;
     const int32_t *tiles;           // point-tile ids of all items
     const int32_t *cta_first;       // [grid + 1]: CTA c runs items [cta_first[c], cta_first[c + 1])
     int n_items;
     int64_t nv;                     // number of valid (sorted) queries
     int nk, metric, K1, S;
-    int stream_a;                   // 1: each stage carries the query tile's K chunk too
+    int list_smem;                  // 1: lists in shared memory while they grow
+    int n_acc;                      // TMEM accumulators
+    int issuers;                    // MMA-issuing threads, 1 or 2
     int64_t n;                      // points
-    float *part_d;                  // [n_items][128][K1]
-    int32_t *part_i;                // [n_items][128][K1]
-    int32_t *part_n;                // [n_items][128]
+    Key *part;                      // [n_items][2 groups][128][K1] ascending lists
+    int32_t *part_n;                // [n_items][2 groups][128] their lengths
     int32_t *err;
     unsigned long long wait_ns;     // limit of a pipeline wait (ESG_BF_WAIT_NS; default 2 s)
     int32_t stall;                  // failure-detection test: the producer first waits on a
@@ -238,8 +313,8 @@ __device__ __forceinline__ bool mbar_try(uint32_t mbar, uint32_t parity) {
 // Bounded wait for the phase of the given parity. Gives up when another role
 // has aborted (unless `ignore_abort`) or after limit_ns; on a timeout it
 // raises the abort flag and the error flag.
-__device__ bool wait_phase(uint32_t mbar, uint32_t parity, volatile int *abort_f, int32_t *err,
-                           unsigned long long limit_ns, bool ignore_abort = false) {
+__device__ __noinline__ bool wait_slow(uint32_t mbar, uint32_t parity, volatile int *abort_f, int32_t *err,
+                                       unsigned long long limit_ns, bool ignore_abort) {
     unsigned long long t0 = 0;
     for (uint32_t it = 1;; ++it) {
         if (mbar_try(mbar, parity)) return true;
@@ -256,6 +331,11 @@ __device__ bool wait_phase(uint32_t mbar, uint32_t parity, volatile int *abort_f
     }
 }
 
+__device__ __forceinline__ bool wait_phase(uint32_t mbar, uint32_t parity, volatile int *abort_f, int32_t *err,
+                                           unsigned long long limit_ns, bool ignore_abort = false) {
+    return mbar_try(mbar, parity) || wait_slow(mbar, parity, abort_f, err, limit_ns, ignore_abort);
+}
+
 __device__ __forceinline__ void mbar_init(uint32_t mbar, uint32_t count) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" :: "r"(mbar), "r"(count) : "memory");
 }
@@ -267,97 +347,156 @@ __device__ __forceinline__ void mbar_arrive(uint32_t mbar) {
 }
 // Bulk global -> shared copy on the TMA engine, completion counted in bytes
 // on the mbarrier (addresses 16-byte aligned, size a multiple of 16).
-__device__ __forceinline__ void bulk_g2s(uint32_t dst, const void *src, uint32_t bytes, uint32_t mbar) {
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                 :: "r"(dst), "l"(src), "r"(bytes), "r"(mbar) : "memory");
+__device__ __forceinline__ void bulk_g2s(uint32_t dst, const void *src, uint32_t bytes, uint32_t mbar, uint64_t hint) {
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1], %2, [%3], %4;"
+                 :: "r"(dst), "l"(src), "r"(bytes), "r"(mbar), "l"(hint) : "memory");
 }
 
-__device__ __forceinline__ void epi_bar() {   // the 256 epilogue threads
-    asm volatile("bar.sync 1, %0;" :: "n"(32 * kEpiWarps) : "memory");
-}
+// What a thread keeps of its row: pending entries, list entries, the list's
+// K1-th distance t and its ceil(K1 / 2)-th distance th (+inf while it is
+// shorter).
+struct RowState {
+    int cnt, len;
+    float t, th;
+};
 
-__device__ __forceinline__ void pair_bar(int quarter) {   // the two warps of a lane quarter
-    asm volatile("bar.sync %0, 64;" :: "r"(2 + quarter) : "memory");
-}
-
-// Lexicographic (distance, row) order of the candidate lists.
-__device__ __forceinline__ bool dl_less(float da, int32_t ia, float db, int32_t ib) {
-    return da < db || (da == db && ia < ib);
-}
-
-// One compare-exchange stage of a bitonic network over 64 (distance, index)
-// pairs, element e = lane + 32 h in (d[h], i[h]); pairs compare by dl_less.
-// Element e meets e ^ j; in a block of size kk that sorts ascending (up) the
-// lower position keeps the smaller pair. `desc` flips every direction.
-__device__ __forceinline__ void bitonic_stage(float (&d)[2], int32_t (&i)[2], int lane, int kk, int j, bool desc) {
-    if (j == 32) {   // partners in the same lane (only in the 64-wide block)
-        const bool sw = desc ? dl_less(d[0], i[0], d[1], i[1]) : dl_less(d[1], i[1], d[0], i[0]);
-        if (sw) {
-            const float td = d[0]; d[0] = d[1]; d[1] = td;
-            const int32_t ti = i[0]; i[0] = i[1]; i[1] = ti;
+// Merges the pending entries of the rows in `mask` (lanes of this warp) into
+// their lists and updates the rows' state (held by lane r for row r); t and th
+// are published as the item tag above the distance's bits. By ranks: lane e
+// holds pending entry e and list entries e + 32 h; each pending entry is read
+// by all lanes in turn (one broadcast), compared with what each lane holds,
+// and a vote counts the list entries before it; then everything is stored at
+// its rank. A sorting network costs the same comparisons but twice the
+// shuffles' and loads' passes through the shared-memory crossbar, of which the
+// MMAs' operand reads and the bulk copies leave little. The next row's entries
+// are loaded meanwhile. Out of line: its call sites are many and rarely taken.
+template <int NL>
+__device__ __noinline__ RowState flush_rows(unsigned mask, const float2 *pend, Key *list, int K1, RowState st,
+                                            volatile Key *pub, uint32_t tag) {
+    const int lane = threadIdx.x & 31;
+    __syncwarp();
+    int r = __ffs(mask) - 1;
+    int c = __shfl_sync(0xffffffffu, st.cnt, r), n = __shfl_sync(0xffffffffu, st.len, r);
+    Key L[NL], p;
+    auto load = [&](int row, int cr, int nr, Key (&l)[NL], Key &q) {
+#pragma unroll
+        for (int h = 0; h < NL; ++h) l[h] = lane + 32 * h < nr ? list[row * K1 + lane + 32 * h] : kPad;
+        q = kPad;
+        if (lane < cr) {
+            const float2 e = pend[lane * kPendStride + row];
+            q = make_key(e.x, __float_as_uint(e.y));
         }
-        return;
+    };
+    load(r, c, n, L, p);
+#pragma unroll 1
+    while (true) {
+        mask &= mask - 1;
+        const int r2 = mask ? __ffs(mask) - 1 : r;
+        const int c2 = __shfl_sync(0xffffffffu, st.cnt, r2), n2 = __shfl_sync(0xffffffffu, st.len, r2);
+        Key L2[NL], p2;
+        if (mask) load(r2, c2, n2, L2, p2);
+        int rp = 0, rl[NL];   // ranks in the merged list
+#pragma unroll
+        for (int h = 0; h < NL; ++h) rl[h] = lane + 32 * h;
+#pragma unroll 4
+        for (int i = 0; i < c; ++i) {
+            const float2 e = pend[i * kPendStride + r];
+            const Key k = make_key(e.x, __float_as_uint(e.y));
+            rp += k < p ? 1 : 0;
+            int below = 0;
+#pragma unroll
+            for (int h = 0; h < NL; ++h) {
+                rl[h] += k < L[h] ? 1 : 0;
+                below += __popc(__ballot_sync(0xffffffffu, L[h] < k));
+            }
+            rp += lane == i ? below : 0;
+        }
+        const int m = min(K1, n + c);
+        const bool pin = lane < c;
+        if (pin && rp < K1) list[r * K1 + rp] = p;
+#pragma unroll
+        for (int h = 0; h < NL; ++h)
+            if (lane + 32 * h < n && rl[h] < K1) list[r * K1 + rl[h]] = L[h];
+        // the distances at rank K1 - 1 and in the middle
+        auto at = [&](int rank) -> float {
+            unsigned b = __ballot_sync(0xffffffffu, pin && rp == rank);
+            uint32_t hi = (uint32_t)(p >> 32);
+#pragma unroll
+            for (int h = 0; h < NL; ++h) {
+                const unsigned bh = __ballot_sync(0xffffffffu, lane + 32 * h < n && rl[h] == rank);
+                if (bh) { b = bh; hi = (uint32_t)(L[h] >> 32); }
+            }
+            return key_dist((Key)__shfl_sync(0xffffffffu, hi, __ffs(b) - 1) << 32);
+        };
+        if (m > (K1 - 1) >> 1) {
+            const float th = at((K1 - 1) >> 1), t = m == K1 ? at(K1 - 1) : INFINITY;
+            if (lane == r) {
+                st.th = th;
+                st.t = t;
+                pub[2 * TM] = ((Key)tag << 32) | __float_as_uint(th);
+                pub[0] = ((Key)tag << 32) | __float_as_uint(t);
+            }
+        }
+        if (lane == r) { st.cnt = 0; st.len = m; }
+        if (!mask) break;
+        r = r2; c = c2; n = n2; p = p2;
+#pragma unroll
+        for (int h = 0; h < NL; ++h) L[h] = L2[h];
     }
+    __syncwarp();
+    return st;
+}
+
+// Inserts the pending entries of every row (one thread each, all rows of the
+// warp together) into the thread's ascending list of KR distances and points:
+// every place takes its old entry, the one before it or the new one, all places
+// at once. Ties keep the earlier entry.
+template <int KR>
+__device__ __forceinline__ void insert_pending(const float2 *pend, int lane, int cnt, float (&d)[KR], int32_t (&id)[KR]) {
+    const int most = __reduce_max_sync(0xffffffffu, cnt);
+#pragma unroll 1
+    for (int i = 0; i < most; ++i) {
+        const float2 e = pend[i * 32 + lane];
+        const float x = i < cnt ? e.x : INFINITY;
+        if (!__any_sync(0xffffffffu, x < d[KR - 1])) continue;   // the list has moved on meanwhile
+        const int32_t xi = __float_as_int(e.y);
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        const float od = __shfl_xor_sync(0xffffffffu, d[h], j);
-        const int32_t oi = __shfl_xor_sync(0xffffffffu, i[h], j);
-        const bool up = (((lane + 32 * h) & kk) == 0) != desc;
-        const bool low = (lane & j) == 0;
-        const bool take = low == up ? dl_less(od, oi, d[h], i[h]) : dl_less(d[h], i[h], od, oi);
-        if (take) { d[h] = od; i[h] = oi; }
+        for (int q = KR - 1; q >= 0; --q) {
+            const bool here = x < d[q], before = q > 0 && x < d[q > 0 ? q - 1 : 0];
+            id[q] = before ? id[q > 0 ? q - 1 : 0] : (here ? xi : id[q]);
+            d[q] = q > 0 ? fminf(d[q], fmaxf(d[q > 0 ? q - 1 : 0], x)) : fminf(d[q], x);
+        }
     }
 }
 
-// Bitonic sort of the 64 pairs (ascending, or descending with `desc`).
-__device__ __forceinline__ void bitonic_sort64(float (&d)[2], int32_t (&i)[2], int lane, bool desc) {
-#pragma unroll
-    for (int kk = 2; kk <= 64; kk <<= 1)
-#pragma unroll
-        for (int j = kk >> 1; j > 0; j >>= 1) bitonic_stage(d, i, lane, kk, j, desc);
-}
-
-// A sorted list (ascending) and 64 sorted candidates (descending), both padded
-// with (+inf, INT32_MAX): the element-wise smaller pairs are the 64 smallest of
-// the union as a bitonic sequence, which one merge pass sorts ascending.
-__device__ __forceinline__ void bitonic_merge_into(float (&ld)[2], int32_t (&li)[2], const float (&cd)[2],
-                                                   const int32_t (&ci)[2], int lane) {
-#pragma unroll
-    for (int h = 0; h < 2; ++h)
-        if (dl_less(cd[h], ci[h], ld[h], li[h])) { ld[h] = cd[h]; li[h] = ci[h]; }
-#pragma unroll
-    for (int j = 32; j > 0; j >>= 1) bitonic_stage(ld, li, lane, 64, j, false);
-}
-
-// Candidates of one row and half tile from which the epilogue sorts and
-// merges them in one network instead of inserting them one at a time (a list
-// that is still filling: the first tile of a work item).
-constexpr int kBulkMin = 32;
-
+// KR > 0: lists of K1 = KR entries in registers; 0: lists of up to 32 NL in memory.
+template <bool L2, int KR, int NL, bool STREAM>
 __global__ void __launch_bounds__(kThreads2, 1) tc_knn2_kernel(Tc2Args a) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    unsigned char *base = (unsigned char *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+    extern __shared__ __align__(1024) unsigned char smem_raw[];
+    constexpr int kPend = KR ? 16 : Epi<STREAM>::kPend, kFill = Epi<STREAM>::kFill;
+    constexpr int kStride = KR ? 32 : kPendStride;   // lists in registers: a slot's 32 rows side by side
     const int K1 = a.K1;
-    // resident query tile: sA holds its nk K chunks for the whole item, a stage
-    // one point chunk; streamed (large d): a stage holds the query chunk and
-    // the point chunk of one K step
-    const int stage_bytes = a.stream_a ? 2 * STAGE : STAGE;
-    unsigned char *sA = base;
-    unsigned char *sB = sA + (a.stream_a ? (size_t)0 : (size_t)a.nk * STAGE);
-    float *T = (float *)(sB + (size_t)a.S * stage_bytes);    // [128][kTS] half tile, transposed
-    float *s_xn = T + TM * kTS;                              // [4 pairs][2][128] tile norms
-    float *L_d = s_xn + 8 * TN;                              // [128][K1] per-row lists
-    int32_t *L_i = (int32_t *)(L_d + TM * K1);
-    int32_t *r_lo = L_i + TM * K1, *r_hi = r_lo + TM, *r_cnt = r_hi + TM, *r_ti = r_cnt + TM;
-    float *r_qn = (float *)(r_ti + TM), *r_td = r_qn + TM;
-    uint32_t *s_flag = (uint32_t *)(r_td + TM);              // [2 halves][4 quarters] row masks
-    uint64_t *bars = (uint64_t *)(s_flag + 8);
+    // tile n of the CTA's run uses accumulator n mod n_acc and barrier n mod
+    // n_bar, an even number: all uses of a barrier belong to one issuer and
+    // one group, so that no one can be a phase ahead of the barrier (with three
+    // barriers for three accumulators, an issuer whose tiles run ahead of the
+    // other's would take an older phase of the same parity for its own)
+    const uint32_t n_acc = (uint32_t)a.n_acc, n_bar = n_acc == 3 ? 6u : n_acc;
+    // a stage: one point chunk, or (streamed) the query chunk and the point
+    // chunk of one K step
+    constexpr int stage_bytes = STREAM ? 2 * STAGE : STAGE;
+    unsigned char *sB = smem_raw;
+    float2 *s_pend = (float2 *)(sB + (size_t)a.S * stage_bytes);   // [8 warps][kPend][kStride]
+    float *s_xn = (float *)(s_pend + kEpiWarps * kPend * kStride);   // [8 warps][128] tile norms
+    Key *s_thr = (Key *)(s_xn + kEpiWarps * TN);             // [K1-th, middle][2 groups][128] published distances
+    uint64_t *bars = (uint64_t *)(s_thr + 4 * TM);
     uint64_t *full = bars, *empty = bars + a.S;
     uint64_t *a_full = bars + 2 * a.S, *a_empty = a_full + 1;
-    uint64_t *acc_full = a_full + 2, *acc_empty = a_full + 4, *drain = a_full + 6;
-    uint32_t *tmem_slot = (uint32_t *)(a_full + 7);
+    uint64_t *acc_full = a_full + 2, *acc_empty = acc_full + 6, *drain = acc_empty + 6;
+    uint64_t *never = drain + 1;                              // nothing arrives on it
+    uint32_t *tmem_slot = (uint32_t *)(never + 1);
     volatile int *abort_f = (volatile int *)(tmem_slot + 1);
-    uint64_t *never = a_full + 8;                             // nothing arrives on it
+    Key *s_list = (Key *)(tmem_slot + 2);                     // [8 warps][32][K1] if list_smem
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     // this CTA's contiguous share of the work items
     const int it_begin = a.cta_first[blockIdx.x];
@@ -368,59 +507,55 @@ __global__ void __launch_bounds__(kThreads2, 1) tc_knn2_kernel(Tc2Args a) {
             mbar_init(smem_u32(full + s), 1);
             mbar_init(smem_u32(empty + s), 1);
         }
-        mbar_init(smem_u32(a_full), 1);
-        mbar_init(smem_u32(a_empty), 1);
-        for (int b = 0; b < 2; ++b) {
+        mbar_init(smem_u32(a_full), kEpiWarps / 2);
+        mbar_init(smem_u32(a_empty), a.issuers);
+        for (int b = 0; b < 6; ++b) {
             mbar_init(smem_u32(acc_full + b), 1);
-            mbar_init(smem_u32(acc_empty + b), kEpiWarps);
+            mbar_init(smem_u32(acc_empty + b), kEpiWarps / 2);
         }
-        mbar_init(smem_u32(drain), 1);
+        mbar_init(smem_u32(drain), a.issuers);
         mbar_init(smem_u32(never), 1);
         *abort_f = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 1) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
-                     :: "r"(smem_u32(tmem_slot)), "r"(2 * TN) : "memory");
+                     :: "r"(smem_u32(tmem_slot)), "r"(kTmem) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
+    for (int i = threadIdx.x; i < 4 * TM; i += kThreads2) s_thr[i] = kPad;   // no item has this tag
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = *tmem_slot;
+    const uint32_t tmem_a = tmem + kTmem - 64 * (uint32_t)a.nk;   // resident query tile: hi chunks, lo chunks
 
     if (warp == 0) {
         if (lane == 0) {
             // ---------------- producer
-            uint32_t s = 0, ps = 0, pa = 0;
+            // operand blocks stream through the L2; lists in global memory stay
+            uint64_t hint;
+            asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(hint));
+            uint32_t s = 0, ps = 0;
             uint32_t issued[kMaxStages] = {0};
             uint32_t ipar[kMaxStages] = {0};
-            bool a_pending = false;
-            uint32_t a_par = 0;
             bool ok = true;
             if (a.stall && !wait_phase(smem_u32(never), 0u, abort_f, a.err, a.wait_ns)) ok = false;
             for (int it = it_begin; ok && it < it_end; ++it) {
                 const WorkItem I = a.items[it];
-                if (!a.stream_a) {
-                    if (!wait_phase(smem_u32(a_empty), pa ^ 1u, abort_f, a.err, a.wait_ns)) { ok = false; break; }
-                    mbar_expect_tx(smem_u32(a_full), (uint32_t)(a.nk * STAGE));
-                    for (int kc = 0; kc < a.nk; ++kc)
-                        bulk_g2s(smem_u32(sA + (size_t)kc * STAGE),
-                                 a.qs + ((int64_t)I.qtile * a.nk + kc) * STAGE, STAGE, smem_u32(a_full));
-                    a_pending = true; a_par = pa;
-                    pa ^= 1u;
-                }
+                int32_t t_nx = a.tiles[I.off];
                 for (int j = 0; ok && j < I.cnt; ++j) {
-                    const int64_t t = a.tiles[I.off + j];
+                    const int64_t t = t_nx;
+                    if (j + 1 < I.cnt) t_nx = __ldg(a.tiles + I.off + j + 1);
                     for (int kc = 0; kc < a.nk; ++kc) {
                         if (!wait_phase(smem_u32(empty + s), ps ^ 1u, abort_f, a.err, a.wait_ns)) { ok = false; break; }
                         unsigned char *sg = sB + (size_t)s * stage_bytes;
                         mbar_expect_tx(smem_u32(full + s), (uint32_t)stage_bytes);
-                        if (a.stream_a) {
+                        if (STREAM) {
                             bulk_g2s(smem_u32(sg), a.qs + ((int64_t)I.qtile * a.nk + kc) * STAGE, STAGE,
-                                     smem_u32(full + s));
+                                     smem_u32(full + s), hint);
                             sg += STAGE;
                         }
-                        bulk_g2s(smem_u32(sg), a.xs + (t * a.nk + kc) * STAGE, STAGE, smem_u32(full + s));
+                        bulk_g2s(smem_u32(sg), a.xs + (t * a.nk + kc) * STAGE, STAGE, smem_u32(full + s), hint);
                         issued[s] = 1; ipar[s] = ps;
                         if (++s == (uint32_t)a.S) { s = 0; ps ^= 1u; }
                     }
@@ -430,282 +565,302 @@ __global__ void __launch_bounds__(kThreads2, 1) tc_knn2_kernel(Tc2Args a) {
                 // let the copies already issued land before the CTA can exit
                 for (int q = 0; q < a.S; ++q)
                     if (issued[q]) wait_phase(smem_u32(full + q), ipar[q], abort_f, a.err, kWaitNs, true);
-                if (a_pending) wait_phase(smem_u32(a_full), a_par, abort_f, a.err, kWaitNs, true);
             }
         }
-    } else if (warp == 1) {
-        if (lane == 0) {
-            // ---------------- MMA issuer
-            uint32_t s = 0, ps = 0, pa = 0, acc_it = 0;
-            uint32_t pacc[2] = {0u, 0u};
+    } else if (warp <= kMmaWarps) {
+        if (lane == 0 && warp <= a.issuers) {
+            // ---------------- MMA issuers: one thread, or two that take the
+            // tiles by parity (a thread's MMAs queue up behind its own waits
+            // and commits, about as long as the MMAs of a stage takes: two
+            // keep the tensor pipe fed)
+            const uint32_t me = (uint32_t)(warp - 1), step = (uint32_t)a.issuers;
+            const uint64_t bdesc0 = sdesc(smem_u32(sB));
+            uint32_t s = me * (uint32_t)a.nk % (uint32_t)a.S, ps = me * (uint32_t)a.nk / (uint32_t)a.S & 1u, pa = 0;
+            uint32_t n = me, n_end = 0, b = me, fb = me;   // tile of the run, its accumulator and barrier
+            // the tile that used the accumulator before: its barrier and phase
+            int before = (int)me - (int)n_acc;
+            uint32_t eb = 0, pe = 0;
             bool ok = true;
             for (int it = it_begin; ok && it < it_end; ++it) {
-                const int cnt = a.items[it].cnt;
-                if (!a.stream_a) {
+                n_end += (uint32_t)a.items[it].cnt;
+                if (!STREAM) {
                     if (!wait_phase(smem_u32(a_full), pa, abort_f, a.err, a.wait_ns)) { ok = false; break; }
                     pa ^= 1u;
                 }
-                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                for (int j = 0; ok && j < cnt; ++j) {
-                    const uint32_t b = acc_it & 1u;
-                    if (!wait_phase(smem_u32(acc_empty + b), pacc[b] ^ 1u, abort_f, a.err, a.wait_ns)) { ok = false; break; }
-                    pacc[b] ^= 1u;
-                    ++acc_it;
-                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                for (; ok && n < n_end; n += step) {
+                    if (before >= 0) {
+                        if (!wait_phase(smem_u32(acc_empty + eb), pe, abort_f, a.err, a.wait_ns)) { ok = false; break; }
+                        if ((eb += step) >= n_bar) { eb -= n_bar; pe ^= 1u; }
+                    } else if ((before += (int)step) >= 0) {
+                        eb = (uint32_t)before;
+                    }
                     const uint32_t dt = tmem + b * TN;
                     for (int kc = 0; kc < a.nk; ++kc) {
                         if (!wait_phase(smem_u32(full + s), ps, abort_f, a.err, a.wait_ns)) { ok = false; break; }
                         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                        const uint32_t sg = smem_u32(sB + (size_t)s * stage_bytes);
-                        const uint32_t ah = a.stream_a ? sg : smem_u32(sA + (size_t)kc * STAGE), al = ah + CHUNK;
-                        const uint32_t bh = a.stream_a ? sg + STAGE : sg, bl = bh + CHUNK;
+                        // descriptors count 16-byte units: 2 per 16 dimensions, CHUNK / 16 from hi to lo
+                        const uint64_t sd = bdesc0 + (uint64_t)(s * (stage_bytes >> 4));
+                        const uint64_t bh = STREAM ? sd + (STAGE >> 4) : sd, bl = bh + (CHUNK >> 4);
+                        const uint32_t first = kc == 0 ? 0u : 1u;
+                        if (STREAM) {
+                            const uint64_t ah = sd, al = sd + (CHUNK >> 4);
 #pragma unroll
-                        for (int st = 0; st < TK / 16; ++st) {
-                            const uint32_t off = st * 32;
-                            mma_bf16(dt, sdesc(ah + off), sdesc(bh + off), (kc == 0 && st == 0) ? 0u : 1u);
-                            mma_bf16(dt, sdesc(ah + off), sdesc(bl + off), 1u);
-                            mma_bf16(dt, sdesc(al + off), sdesc(bh + off), 1u);
+                            for (int st = 0; st < TK / 16; ++st) {
+                                mma_bf16(dt, ah + 2 * st, bh + 2 * st, st == 0 ? first : 1u);
+                                mma_bf16(dt, ah + 2 * st, bl + 2 * st, 1u);
+                                mma_bf16(dt, al + 2 * st, bh + 2 * st, 1u);
+                            }
+                        } else {
+                            const uint32_t ah = tmem_a + kc * 32, al = ah + a.nk * 32;
+#pragma unroll
+                            for (int st = 0; st < TK / 16; ++st) {
+                                mma_bf16_ta(dt, ah + st * 8, bh + 2 * st, st == 0 ? first : 1u);
+                                mma_bf16_ta(dt, ah + st * 8, bl + 2 * st, 1u);
+                                mma_bf16_ta(dt, al + st * 8, bh + 2 * st, 1u);
+                            }
                         }
                         mma_commit(smem_u32(empty + s));
                         if (++s == (uint32_t)a.S) { s = 0; ps ^= 1u; }
                     }
-                    if (ok) mma_commit(smem_u32(acc_full + b));
+                    if (!ok) break;
+                    mma_commit(smem_u32(acc_full + fb));
+                    if ((b += step) >= n_acc) b -= n_acc;
+                    if ((fb += step) >= n_bar) fb -= n_bar;
+                    if (step == 2)   // past the other issuer's tile
+                        for (s += (uint32_t)a.nk; s >= (uint32_t)a.S; s -= (uint32_t)a.S) ps ^= 1u;
                 }
-                if (ok && !a.stream_a) mma_commit(smem_u32(a_empty));
+                if (ok && !STREAM) mma_commit(smem_u32(a_empty));
             }
             // all MMAs issued by this thread complete before the CTA exits
             mma_commit(smem_u32(drain));
             wait_phase(smem_u32(drain), 0u, abort_f, a.err, kWaitNs, true);
         }
     } else {
-        // ---------------- epilogue (256 threads, 4 pairs of warps)
-        // The two warps of a pair read the same 32 TMEM lanes (rows), one
-        // column half each, and are the only ones to touch those rows' state:
-        // within a tile they synchronise with a 64-thread barrier of their
-        // own. Block-wide barriers remain only where rows change hands (a new
-        // query tile, the write-out). After an aborted wait the loops still
-        // run to the end (every wait then returns at once), so that all
-        // threads meet the same barriers; the host reports the error.
-        const int ew = warp - 2;            // 0..7
-        const int et = ew * 32 + lane;      // 0..255
+        // ---------------- epilogue
+        const int ew = warp - 1 - kMmaWarps;   // 0..7
+        const int group = ew >> 2;          // takes the tiles of this parity
         const int quarter = warp & 3;       // TMEM lanes this warp may read
-        const int half = ew >> 2;           // column half it reads
-        const int pt_i = half * 32 + lane;  // thread index within the pair
         const int my_row = quarter * 32 + lane;
-        const bool l2 = a.metric == ESG_L2SQ;
-        uint32_t acc_it = 0, tcount = 0;
-        uint32_t pe[2] = {0u, 0u};
-        int cur_qt = -1;
-        // squared norms of a tile into the pair's buffer
-        auto load_norms = [&](int32_t tile, float *dst) {
-            if (!l2) return;
-            const int32_t p0 = tile * TN + pt_i, p1 = p0 + 64;
-            dst[pt_i] = p0 < a.n ? __ldg(a.xnorm + p0) : 0.f;
-            dst[pt_i + 64] = p1 < a.n ? __ldg(a.xnorm + p1) : 0.f;
-        };
+        float2 *pend = s_pend + ew * kPend * kStride;
+        float *xs = s_xn + ew * TN;
+        constexpr uint32_t kSlotBytes = sizeof(float2) * kStride;
+        const uint32_t slot0 = smem_u32(pend + lane);   // the row's first pending slot
+        volatile Key *pub = s_thr + group * TM + my_row;   // K1-th distance; the middle one 2 TM further
+        volatile const Key *pub_o = s_thr + (1 - group) * TM + my_row;
+        uint32_t pa = 0, b = (uint32_t)group, fb = (uint32_t)group, pf = 0;   // accumulator, barrier and its phase
         // the CTA's items are consecutive pieces of the covered-tile sequence,
-        // so its tiles are one run a.tiles[g_beg, g_end): the index of the
-        // tile after next and the next tile's norms are fetched into
-        // registers a tile ahead of their use
+        // so its tiles are one run a.tiles[g_beg, g_end) and tile n of the run
+        // is accumulator use n; the index of the group's tile after next and
+        // the next tile's norms are fetched into registers ahead of their use
         const int32_t g_beg = it_begin < it_end ? a.items[it_begin].off : 0;
-        const int32_t g_end = it_begin < it_end ? a.items[it_end - 1].off + a.items[it_end - 1].cnt : 0;
-        int32_t g_cur = g_beg;
-        int32_t tile_cur = g_beg < g_end ? a.tiles[g_beg] : 0;
-        int32_t tile_nx = g_beg + 1 < g_end ? a.tiles[g_beg + 1] : -1;
-        if (g_beg < g_end) load_norms(tile_cur, s_xn + (quarter * 2) * TN);
-        for (int it = it_begin; it < it_end; ++it) {
+        const int32_t g_n = it_begin < it_end ? a.items[it_end - 1].off + a.items[it_end - 1].cnt - g_beg : 0;
+        int32_t n = group;
+        int32_t tile_cur = n < g_n ? a.tiles[g_beg + n] : 0;
+        int32_t tile_nx = n + 2 < g_n ? a.tiles[g_beg + n + 2] : 0;
+        float4 xn = make_float4(0.f, 0.f, 0.f, 0.f);   // norms 4 lane .. 4 lane + 3 of the tile
+        if (L2 && n < g_n) xn = __ldg((const float4 *)(a.xnorm + (int64_t)tile_cur * TN) + lane);
+        bool ok = true;
+        for (int it = it_begin; ok && it < it_end; ++it) {
             const WorkItem I = a.items[it];
-            if (I.qtile != cur_qt) {
-                // new query tile: per-row state (the lists of the previous tile
-                // were written out at the end of its last item)
-                if (et < TM) {
-                    const int64_t sp = (int64_t)I.qtile * TM + et;
-                    int32_t lo = 1, hi = 0;
-                    float qn = 0.f;
-                    if (sp < a.nv) {
-                        const int32_t o = a.qorder[sp];
-                        lo = (int32_t)a.l[o]; hi = (int32_t)a.r[o];
-                        if (l2) qn = a.qnorm[o];
+            const int32_t n_end = I.off + I.cnt - g_beg;
+            if (!STREAM && group == 0) {
+                // the item's query tile into tensor memory, once the MMAs of
+                // the previous item are done: each thread its row, 64 hi and
+                // 64 lo BF16 (32 columns each) per chunk
+                if (!wait_phase(smem_u32(a_empty), pa ^ 1u, abort_f, a.err, a.wait_ns)) {
+                    ok = false;
+                } else {
+                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                    for (int h = 0; h < 2 * a.nk; ++h) {
+                        const int kc = h >> 1, lo_part = h & 1;
+                        const unsigned char *src = a.qs + ((int64_t)I.qtile * a.nk + kc) * STAGE + lo_part * CHUNK +
+                                                   my_row * 128;
+                        uint4 w[8];
+#pragma unroll
+                        for (int c = 0; c < 8; ++c) w[c] = __ldg((const uint4 *)(src + ((c ^ (my_row & 7)) << 4)));
+                        tmem_st32(tmem_a + ((uint32_t)(quarter * 32) << 16) + (lo_part * a.nk + kc) * 32, w);
                     }
-                    r_lo[et] = lo; r_hi[et] = hi; r_qn[et] = qn;
-                    r_cnt[et] = 0; r_td[et] = INFINITY; r_ti[et] = 0x7FFFFFFF;
+                    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+                    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(smem_u32(a_full));
+                    pa ^= 1u;
                 }
-                cur_qt = I.qtile;
-                epi_bar();
             }
-            for (int j = 0; j < I.cnt; ++j, ++g_cur) {
+            Key *out = a.part + (((int64_t)it * 2 + group) * TM + quarter * 32) * K1;
+            Key *list = a.list_smem ? s_list + ew * 32 * K1 : out;
+            const int64_t sp = (int64_t)I.qtile * TM + my_row;
+            int32_t lo = 1, hi = 0;
+            float *drow = nullptr;   // a dense row's distance of point p goes to drow[p]
+            if (sp < a.nv) {
+                const int32_t o = a.qorder[sp];
+                // a query whose norm overflows keeps no candidates
+                if (!L2 || a.qnorm[o] < INFINITY) { lo = (int32_t)a.l[o]; hi = (int32_t)a.r[o]; }
+                const int64_t off = a.doff[sp];
+                if (off >= 0) drow = a.dense + off - (lo & ~3);
+            }
+            RowState st{0, 0, INFINITY, INFINITY};   // points at +inf or NaN are never kept
+            constexpr int KL = KR ? KR : 1;
+            float ld[KL];
+            int32_t li[KL];
+#pragma unroll
+            for (int e = 0; e < KL; ++e) { ld[e] = INFINITY; li[e] = 0; }
+            // all pending entries of the warp's rows (those worth it, with
+            // lists in memory) into their lists
+            auto flush = [&](int fill) {
+                if constexpr (KR > 0) {
+                    __syncwarp();
+                    insert_pending<KL>(pend, lane, st.cnt, ld, li);
+                    __syncwarp();
+                    st.cnt = 0;
+                    st.t = ld[KL - 1];
+                    st.th = ld[(KL - 1) / 2];
+                    pub[0] = ((Key)(uint32_t)it << 32) | __float_as_uint(st.t);
+                    pub[2 * TM] = ((Key)(uint32_t)it << 32) | __float_as_uint(st.th);
+                } else if constexpr (KR == 0) {
+                    const unsigned fl = __ballot_sync(0xffffffffu, st.cnt >= fill);
+                    if (fl) st = flush_rows<NL>(fl, pend, list, K1, st, pub, (uint32_t)it);
+                }
+            };
+            for (; ok && n < n_end; n += 2) {
                 const int32_t pt = tile_cur * TN;   // first point of the tile
-                float *xs_cur = s_xn + (quarter * 2 + (tcount & 1u)) * TN;
-                // the next tile's norms (stored after the filter into the
-                // pair's other buffer, whose last readers finished before the
-                // previous tile's pair barriers) and the index after it
-                float *xs_nx = s_xn + (quarter * 2 + ((tcount + 1u) & 1u)) * TN;
-                float xn_a = 0.f, xn_b = 0.f;
-                if (l2 && tile_nx >= 0) {
-                    const int32_t p0 = tile_nx * TN + pt_i, p1 = p0 + 64;
-                    xn_a = p0 < a.n ? __ldg(a.xnorm + p0) : 0.f;
-                    xn_b = p1 < a.n ? __ldg(a.xnorm + p1) : 0.f;
+                if (L2) {
+                    ((float4 *)xs)[lane] = xn;
+                    __syncwarp();
+                    if (n + 2 < g_n) xn = __ldg((const float4 *)(a.xnorm + (int64_t)tile_nx * TN) + lane);
                 }
-                const int32_t tile_nx2 = g_cur + 2 < g_end ? __ldg(a.tiles + g_cur + 2) : -1;
-                ++tcount;
-                const uint32_t b = acc_it & 1u;
-                wait_phase(smem_u32(acc_full + b), pe[b], abort_f, a.err, a.wait_ns);
-                pe[b] ^= 1u;
-                ++acc_it;
+                const int32_t tile_nx2 = n + 4 < g_n ? __ldg(a.tiles + g_beg + n + 4) : 0;
+                if (!wait_phase(smem_u32(acc_full + fb), pf, abort_f, a.err, a.wait_ns)) {
+                    ok = false;
+                    break;
+                }
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                // the row's range within this half tile; a warp none of whose
-                // 32 rows covers it skips the accumulator load and the filter
-                const int32_t pbm = pt + half * 64;
-                const int32_t lo = r_lo[my_row], hi = r_hi[my_row];
-                const int jl = lo - pbm > 0 ? lo - pbm : 0;
-                const int jh = hi - pbm < 63 ? hi - pbm : 63;
-                const uint64_t rng = jl <= jh ? ((~0ull >> (63 - (jh - jl))) << jl) : 0ull;
-                const bool warp_in = __any_sync(0xffffffffu, rng != 0ull);
-                float v[64];
-                if (warp_in) tmem_ld64(tmem + ((uint32_t)(quarter * 32) << 16) + b * TN + half * 64, v);
-                asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-                __syncwarp();
-                if (lane == 0) mbar_arrive(smem_u32(acc_empty + b));
-                // filter, one thread per row and half: distances of the 64
-                // columns, range mask, and the columns at or below the row's
-                // current K1-th distance (a superset of the insertions)
-                uint64_t cand = 0ull;
-                if (warp_in) {
-                    const float qn = r_qn[my_row], tdm = r_td[my_row];
-                    const float4 *xv = (const float4 *)(xs_cur + half * 64);
+                // the row's columns jl..jh of this tile; a warp none of whose
+                // rows covers it only releases the accumulator
+                const int jl = lo - pt > 0 ? lo - pt : 0;
+                const int jh = hi - pt < TN - 1 ? hi - pt : TN - 1;
+                const bool in = jl <= jh;
+                auto release = [&]() {   // the accumulator is read
+                    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(smem_u32(acc_empty + fb));
+                };
+                if (__any_sync(0xffffffffu, in)) {
+                    const bool masked = !__all_sync(0xffffffffu, !in || jh - jl == TN - 1);
+                    const Key o = pub_o[0], oh = pub_o[2 * TM];
+                    const float to = (uint32_t)(o >> 32) == (uint32_t)it ? __uint_as_float((uint32_t)o) : INFINITY;
+                    const float tho = (uint32_t)(oh >> 32) == (uint32_t)it ? __uint_as_float((uint32_t)oh) : INFINITY;
+                    const bool lists = in && drow == nullptr;
+                    const bool any_dense = __any_sync(0xffffffffu, in && drow != nullptr);
+                    float thr = lists ? fminf(fminf(st.t, to), fmaxf(st.th, tho)) : -INFINITY;
+                    const uint32_t ta = tmem + ((uint32_t)(quarter * 32) << 16) + b * TN;
+                    uint32_t slot = slot0 + st.cnt * kSlotBytes;
+#pragma unroll 1
+                    for (int c0 = 0; c0 < TN; c0 += 32) {
+                        float s[32];
+                        // the columns' distances |x|^2 - 2 q.x (the query's own
+                        // norm, the same for every point, is left out) or
+                        // -q.x, +inf outside the row's range, and the least of
+                        // each kCols: most blocks hold nothing for any row
+                        if (L2) {
+                            float4 x[8];
 #pragma unroll
-                    for (int c4 = 0; c4 < 16; ++c4) {
-                        const float4 x4 = xv[c4];
-                        const float xx[4] = {x4.x, x4.y, x4.z, x4.w};
+                            for (int c = 0; c < 8; ++c) x[c] = *(const float4 *)(xs + c0 + 4 * c);
+                            tmem_ld32(ta + c0, s);
+                            if (c0 == TN - 32) release();
 #pragma unroll
-                        for (int e = 0; e < 4; ++e) {
-                            const int c = c4 * 4 + e;
-                            const float dd = l2 ? qn + xx[e] - 2.f * v[c] : -v[c];
-                            v[c] = dd;
-                            cand |= (uint64_t)(dd <= tdm) << c;
-                        }
-                    }
-                    cand &= rng;
-                }
-                if (l2 && tile_nx >= 0) { xs_nx[pt_i] = xn_a; xs_nx[pt_i + 64] = xn_b; }
-                const bool fl = cand != 0ull;
-                const uint32_t wm = __ballot_sync(0xffffffffu, fl);
-                if (lane == 0) s_flag[half * 4 + quarter] = wm;
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    // flagged rows of this half pass their distances through
-                    // shared memory (out-of-range columns as +inf)
-                    if (half == h && fl) {
-#pragma unroll
-                        for (int c = 0; c < 64; ++c)
-                            T[my_row * kTS + c] = ((rng >> c) & 1ull) ? v[c] : INFINITY;
-                    }
-                    pair_bar(quarter);
-                    // warp-cooperative insertion: the k-th flagged row of the
-                    // pair's 32 goes to the pair's warp k mod 2
-                    const int32_t pb = pt + h * 64;
-                    uint32_t w = s_flag[h * 4 + quarter];
-                    int k = 0;
-                    while (w != 0u) {
-                        const int bit = __ffs(w) - 1;
-                        w &= w - 1;
-                        if ((k++ & 1) != half) continue;
-                        const int r = quarter * 32 + bit;
-                        const int32_t p0 = pb + lane, p1 = p0 + 32;
-                        const float d0 = T[r * kTS + lane], d1 = T[r * kTS + lane + 32];
-                        float td = r_td[r];
-                        int32_t ti = r_ti[r];
-                        uint32_t m0 = __ballot_sync(0xffffffffu, d0 < INFINITY && dl_less(d0, p0, td, ti));
-                        uint32_t m1 = __ballot_sync(0xffffffffu, d1 < INFINITY && dl_less(d1, p1, td, ti));
-                        if ((m0 | m1) == 0u) continue;                  // warp-uniform
-                        // the row's list in registers: entries lane and lane + 32
-                        int cnt = r_cnt[r];
-                        float ld0 = lane < cnt ? L_d[r * K1 + lane] : INFINITY;
-                        int32_t li0 = lane < cnt ? L_i[r * K1 + lane] : 0x7FFFFFFF;
-                        float ld1 = lane + 32 < cnt ? L_d[r * K1 + lane + 32] : INFINITY;
-                        int32_t li1 = lane + 32 < cnt ? L_i[r * K1 + lane + 32] : 0x7FFFFFFF;
-                        const int nc = __popc(m0) + __popc(m1);
-                        if (nc >= kBulkMin) {
-                            // the K1 smallest of list and candidates in one
-                            // network: the same list as inserting one by one
-                            const bool in0 = (m0 >> lane) & 1u, in1 = (m1 >> lane) & 1u;
-                            float cd[2] = {in0 ? d0 : INFINITY, in1 ? d1 : INFINITY};
-                            int32_t ci[2] = {in0 ? p0 : 0x7FFFFFFF, in1 ? p1 : 0x7FFFFFFF};
-                            bitonic_sort64(cd, ci, lane, true);
-                            float ld[2] = {ld0, ld1};
-                            int32_t li[2] = {li0, li1};
-                            bitonic_merge_into(ld, li, cd, ci, lane);
-                            ld0 = ld[0]; li0 = li[0]; ld1 = ld[1]; li1 = li[1];
-                            cnt = min(K1, cnt + nc);
-                            if (cnt == K1) {
-                                const int e = K1 - 1;
-                                td = __shfl_sync(0xffffffffu, e < 32 ? ld0 : ld1, e & 31);
-                                ti = __shfl_sync(0xffffffffu, e < 32 ? li0 : li1, e & 31);
+                            for (int c = 0; c < 8; ++c) {
+                                s[4 * c] = fmaf(-2.f, s[4 * c], x[c].x);
+                                s[4 * c + 1] = fmaf(-2.f, s[4 * c + 1], x[c].y);
+                                s[4 * c + 2] = fmaf(-2.f, s[4 * c + 2], x[c].z);
+                                s[4 * c + 3] = fmaf(-2.f, s[4 * c + 3], x[c].w);
                             }
-                            m0 = m1 = 0u;
+                        } else {
+                            tmem_ld32(ta + c0, s);
+                            if (c0 == TN - 32) release();
+#pragma unroll
+                            for (int c = 0; c < 32; ++c) s[c] = -s[c];
                         }
-                        while ((m0 | m1) != 0u) {
-                            const bool second = m0 == 0u;
-                            const int src = __ffs(second ? m1 : m0) - 1;
-                            if (second) m1 &= m1 - 1; else m0 &= m0 - 1;
-                            const float cd = __shfl_sync(0xffffffffu, second ? d1 : d0, src);
-                            const int32_t ci = pb + (second ? 32 : 0) + src;
-                            if (cnt == K1 && !dl_less(cd, ci, td, ti)) continue;
-                            const int pos = __popc(__ballot_sync(0xffffffffu, lane < cnt && dl_less(ld0, li0, cd, ci))) +
-                                            __popc(__ballot_sync(0xffffffffu, lane + 32 < cnt && dl_less(ld1, li1, cd, ci)));
-                            const float u0d = __shfl_up_sync(0xffffffffu, ld0, 1);
-                            const int32_t u0i = __shfl_up_sync(0xffffffffu, li0, 1);
-                            float u1d = __shfl_up_sync(0xffffffffu, ld1, 1);
-                            int32_t u1i = __shfl_up_sync(0xffffffffu, li1, 1);
-                            const float t31d = __shfl_sync(0xffffffffu, ld0, 31);
-                            const int32_t t31i = __shfl_sync(0xffffffffu, li0, 31);
-                            if (lane == 0) { u1d = t31d; u1i = t31i; }
-                            if (lane > pos) { ld0 = u0d; li0 = u0i; }
-                            else if (lane == pos) { ld0 = cd; li0 = ci; }
-                            if (lane + 32 > pos) { ld1 = u1d; li1 = u1i; }
-                            else if (lane + 32 == pos) { ld1 = cd; li1 = ci; }
-                            if (cnt < K1) ++cnt;
-                            if (cnt == K1) {
-                                const int e = K1 - 1;
-                                td = __shfl_sync(0xffffffffu, e < 32 ? ld0 : ld1, e & 31);
-                                ti = __shfl_sync(0xffffffffu, e < 32 ? li0 : li1, e & 31);
+                        if (masked) {
+#pragma unroll
+                            for (int c = 0; c < 32; ++c)
+                                s[c] = (uint32_t)(c0 + c - jl) <= (uint32_t)(jh - jl) ? s[c] : INFINITY;
+                        }
+                        if (any_dense) {
+#pragma unroll
+                            for (int c = 0; c < 32; c += 4)
+                                if (in && drow != nullptr && c0 + c + 3 >= jl && c0 + c <= jh)
+                                    *(float4 *)(drow + pt + c0 + c) = make_float4(s[c], s[c + 1], s[c + 2], s[c + 3]);
+                        }
+                        float least[32 / kCols];
+#pragma unroll
+                        for (int g = 0; g < 32 / kCols; ++g) {
+                            const float *t8 = s + g * kCols;
+                            least[g] = fminf(fminf(fminf(t8[0], t8[1]), fminf(t8[2], t8[3])),
+                                             fminf(fminf(t8[4], t8[5]), fminf(t8[6], t8[7])));
+                        }
+                        if (!__any_sync(0xffffffffu, fminf(fminf(least[0], least[1]), fminf(least[2], least[3])) < thr))
+                            continue;
+#pragma unroll
+                        for (int g = 0; g < 32 / kCols; ++g) {
+                            if (!__any_sync(0xffffffffu, least[g] < thr)) continue;
+                            // predicated, not branches: the candidates are
+                            // spread over the warp's rows
+#pragma unroll
+                            for (int c = g * kCols; c < (g + 1) * kCols; ++c)
+                                asm volatile(
+                                    "{\n\t.reg .pred p;\n\tsetp.lt.f32 p, %1, %2;\n\t"
+                                    "@p st.shared.v2.b32 [%0], {%3, %4};\n\t@p add.u32 %0, %0, %5;\n\t}\n"
+                                    : "+r"(slot)
+                                    : "f"(s[c]), "f"(thr), "r"(__float_as_uint(s[c])), "r"(pt + c0 + c),
+                                      "n"(kSlotBytes)
+                                    : "memory");
+                            if (__any_sync(0xffffffffu, slot > slot0 + (kPend - kCols) * kSlotBytes)) {
+                                st.cnt = (int)((slot - slot0) / kSlotBytes);
+                                flush(kFill);
+                                slot = slot0 + st.cnt * kSlotBytes;
+                                thr = lists ? fminf(fminf(st.t, to), fmaxf(st.th, tho)) : -INFINITY;
                             }
                         }
-                        if (lane < cnt) { L_d[r * K1 + lane] = ld0; L_i[r * K1 + lane] = li0; }
-                        if (lane + 32 < cnt) { L_d[r * K1 + lane + 32] = ld1; L_i[r * K1 + lane + 32] = li1; }
-                        if (lane == 0) { r_cnt[r] = cnt; r_td[r] = td; r_ti[r] = ti; }
-                        __syncwarp();
                     }
-                    pair_bar(quarter);
+                    st.cnt = (int)((slot - slot0) / kSlotBytes);
                 }
+                else release();
+                if ((b += 2) >= n_acc) b -= n_acc;
+                if ((fb += 2) >= n_bar) { fb -= n_bar; pf ^= 1u; }
                 tile_cur = tile_nx;
                 tile_nx = tile_nx2;
             }
-            // write the lists out when this is the CTA's last item of the
-            // query tile (a row's list then covers all of the tile's items
-            // this CTA ran); other items record empty lists
-            const bool flush = it + 1 == it_end || a.items[it + 1].qtile != I.qtile;
-            if (flush) epi_bar();   // every pair's insertions are done
-            for (int r = et; r < TM; r += 32 * kEpiWarps) {
-                const int c = flush ? r_cnt[r] : 0;
-                a.part_n[(int64_t)it * TM + r] = c;
+            if (!ok) {   // an aborted wait: no lists (the host reports the error)
+                for (; it < it_end; ++it) a.part_n[((int64_t)it * 2 + group) * TM + my_row] = 0;
+                break;
             }
-            if (flush) {
-                for (int idx = et; idx < TM * K1; idx += 32 * kEpiWarps) {
-                    const int r = idx / K1, e = idx % K1;
-                    if (e < r_cnt[r]) {
-                        a.part_d[(int64_t)it * TM * K1 + idx] = L_d[idx];
-                        a.part_i[(int64_t)it * TM * K1 + idx] = L_i[idx];
+            __syncwarp();
+            flush(1);
+            if (KR) {
+#pragma unroll
+                for (int e = 0; e < KL; ++e) {
+                    if (ld[e] < INFINITY) {
+                        out[(size_t)lane * KL + e] = make_key(ld[e], (uint32_t)li[e]);
+                        st.len = e + 1;
                     }
                 }
-                epi_bar();
+            } else if (a.list_smem) {
+                for (int r = 0; r < 32; ++r) {
+                    const int m = __shfl_sync(0xffffffffu, st.len, r);
+#pragma unroll
+                    for (int h = 0; h < NL; ++h)
+                        if (lane + 32 * h < m) out[(size_t)r * K1 + lane + 32 * h] = list[r * K1 + lane + 32 * h];
+                }
+                __syncwarp();
             }
+            a.part_n[((int64_t)it * 2 + group) * TM + my_row] = st.len;
         }
     }
     __syncthreads();
     if (warp == 1) {
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(tmem), "r"(2 * TN) : "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(tmem), "r"(kTmem) : "memory");
     }
 }
 
@@ -791,110 +946,276 @@ cudaError_t split_norm(const float *X, int64_t rows, int d, int nk, const int32_
     return cudaGetLastError();
 }
 
-// Merge the per-item top-K1 lists of each valid query (one warp per sorted
-// position) into one top-K1 list in the caller's query order. Lists are
-// ascending in (distance, row) and hold distinct rows, so the position of
-// an element in the merged list is its own index plus the number of
-// elements of the other list that precede it.
-__global__ void merge_parts_kernel(const float *part_d, const int32_t *part_i, const int32_t *part_n,
-                                   const int32_t *item_begin, const int32_t *qorder, int64_t nv, int K1,
-                                   float *cand_d, int32_t *cand_i, int32_t *cand_n) {
-    __shared__ Cand buf[4][3][kMaxK1v2];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int64_t sp = blockIdx.x * (int64_t)4 + w;
-    if (sp >= nv) return;
+struct FinishArgs {
+    const float *X, *Q;
+    int d, metric, k, K1;
+    const Key *part;
+    const int32_t *part_n, *item_begin, *qorder;
+    const int64_t *doff, *l, *r;
+    const float *dense;
+    const float *qnorm, *qrownorm, *xmax;
+    int64_t *out_ids;
+    float *out_dist;
+    int32_t *out_count, *redo;
+};
+
+// One valid query per block of WQ warps, at its sorted position: its lists
+// (two per work item of its query tile) merged into the K1 best approximate
+// distances, each warp every WQ-th list, then the warps' results pairwise;
+// the candidates' exact FP32 distances, four per warp at a time; sort,
+// certificate and output by warp 0. All keys stay in registers (32 NL per
+// list). A block per query because the lists and the candidates' rows are
+// dependent gathers: a warp per query took the 304 lists of a 61-query call in
+// series (208 us) and one candidate row after the other (40 us). WQ: 4, or 16
+// when the queries' lists are many (few queries over many CTAs).
+// Together 57 us for 10k queries of lists, 300 us with 0.9 GB of dense rows.
+template <int NL, int WQ>
+__global__ void __launch_bounds__(32 * WQ) finish_kernel(FinishArgs f) {
+    __shared__ Key s_keys[WQ][32 * NL];
+    __shared__ int s_na[WQ];
+    __shared__ Key s_buf[WQ][32 + 256];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t sp = blockIdx.x;
     const int64_t qt = sp / TM;
     const int row = (int)(sp % TM);
-    Cand *A = buf[w][0], *B = buf[w][1], *C = buf[w][2];
+    const int64_t q = f.qorder[sp];
+    const int l0 = f.item_begin[qt] * 2, l1 = f.item_begin[qt + 1] * 2;
+    Key A[NL];
+#pragma unroll
+    for (int h = 0; h < NL; ++h) A[h] = kPad;
     int na = 0;
-    for (int it = item_begin[qt]; it < item_begin[qt + 1]; ++it) {
-        const int64_t sub = (int64_t)it * TM + row;
-        const int nb = part_n[sub];
-        if (nb <= 0) continue;
-        for (int e = lane; e < nb; e += 32)
-            B[e] = Cand{part_d[sub * K1 + e], (uint32_t)part_i[sub * K1 + e]};
-        __syncwarp();
-        for (int i = lane; i < na; i += 32) {
-            int lo = 0, hi = nb;   // number of B elements before A[i]
-            while (lo < hi) {
-                const int m = (lo + hi) >> 1;
-                if (cand_less(B[m].d, B[m].id, A[i].d, A[i].id)) lo = m + 1; else hi = m;
+    const int64_t off = f.doff[sp];
+    if (off >= 0) {
+        // a dense row: each warp takes every WQ-th 128 distances; those below
+        // its K1-th so far are collected, and sorted and merged by 32
+        const int32_t lo = (int32_t)f.l[q], hi = (int32_t)f.r[q];
+        const float4 *row = (const float4 *)(f.dense + off);
+        const bool dead = f.metric == ESG_L2SQ && !(f.qnorm[q] < INFINITY);
+        Key *buf = s_buf[warp];
+        int nb = 0;
+        float t = INFINITY;
+        auto merge32 = [&](int c) {
+            Key p[NL];
+#pragma unroll
+            for (int h = 0; h < NL; ++h) p[h] = kPad;
+            if (lane < c) p[0] = buf[lane];
+            Key one[1] = {p[0]};
+            sort_asc<1>(one, lane);
+            p[0] = one[0];
+            merge_lists<NL>(A, p, lane);
+            na = min(f.K1, na + c);
+            Key k = kPad;
+#pragma unroll
+            for (int h = 0; h < NL; ++h)
+                if (h == (f.K1 - 1) >> 5) k = A[h];
+            k = __shfl_sync(0xffffffffu, k, (f.K1 - 1) & 31);
+            if (na == f.K1) t = key_dist(k);
+        };
+        const int32_t p0 = lo & ~3;
+        const float4 none = make_float4(INFINITY, INFINITY, INFINITY, INFINITY);
+        for (int32_t c0 = dead ? hi + 1 : p0 + 256 * warp; c0 <= hi; c0 += 256 * WQ) {
+            const int32_t pt = c0 + 4 * lane;
+            const float4 xa = pt <= hi ? row[(pt - p0) >> 2] : none;
+            const float4 xb = pt + 128 <= hi ? row[(pt + 128 - p0) >> 2] : none;
+            const float x[8] = {xa.x, xa.y, xa.z, xa.w, xb.x, xb.y, xb.z, xb.w};
+            const float least = fminf(fminf(fminf(x[0], x[1]), fminf(x[2], x[3])),
+                                      fminf(fminf(x[4], x[5]), fminf(x[6], x[7])));
+            if (!__any_sync(0xffffffffu, least < t)) continue;
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                const int32_t p = pt + (e < 4 ? e : 124 + e);
+                const bool take = x[e] < t && p >= lo && p <= hi;
+                const unsigned b = __ballot_sync(0xffffffffu, take);
+                if (b == 0u) continue;
+                if (take) buf[nb + __popc(b & ((1u << lane) - 1))] = make_key(x[e], (uint32_t)p);
+                nb += __popc(b);
             }
-            if (i + lo < K1) C[i + lo] = A[i];
-        }
-        for (int j = lane; j < nb; j += 32) {
-            int lo = 0, hi = na;   // number of A elements before B[j]
-            while (lo < hi) {
-                const int m = (lo + hi) >> 1;
-                if (cand_less(A[m].d, A[m].id, B[j].d, B[j].id)) lo = m + 1; else hi = m;
+            __syncwarp();
+            while (nb >= 32) {
+                merge32(32);
+                __syncwarp();
+                nb -= 32;   // the last 32 in the place of those merged
+                const int mv = min(nb, 32);
+                if (lane < mv) buf[lane] = buf[32 + nb - mv + lane];
+                __syncwarp();
             }
-            if (j + lo < K1) C[j + lo] = B[j];
         }
-        __syncwarp();
-        Cand *t = A; A = C; C = t;
-        na = min(K1, na + nb);
+        if (nb > 0) merge32(nb);
+    } else for (int li = l0 + warp; li < l1; li += WQ) {
+        const int64_t sub = (int64_t)li * TM + row;
+        const int nb = f.part_n[sub];
+        Key B[NL];
+#pragma unroll
+        for (int h = 0; h < NL; ++h) {
+            const int e = lane + 32 * h;
+            B[h] = e < f.K1 ? f.part[sub * f.K1 + e] : kPad;   // entries past nb are not written: dropped below
+            if (e >= nb) B[h] = kPad;
+        }
+        if (nb == 0) continue;
+        merge_lists<NL>(A, B, lane);
+        na = min(f.K1, na + nb);
     }
-    const int32_t o = qorder[sp];
-    for (int e = lane; e < na; e += 32) {
-        cand_d[(int64_t)o * K1 + e] = A[e].d;
-        cand_i[(int64_t)o * K1 + e] = (int32_t)A[e].id;
+#pragma unroll
+    for (int w = WQ / 2; w > 0; w >>= 1) {   // warps w .. 2w - 1 hand their lists to warps 0 .. w - 1
+        if (warp >= w && warp < 2 * w) {
+#pragma unroll
+            for (int h = 0; h < NL; ++h) s_keys[warp][lane + 32 * h] = A[h];
+            if (lane == 0) s_na[warp] = na;
+        }
+        __syncthreads();
+        if (warp < w && s_na[warp + w] > 0) {
+#pragma unroll
+            for (int h = 0; h < NL; ++h)
+                A[h] = key_min(A[h], s_keys[warp + w][32 * NL - 1 - (lane + 32 * h)]);
+            bitonic_asc<NL>(A, lane);
+            na = min(f.K1, na + s_na[warp + w]);
+        }
     }
-    if (lane == 0) cand_n[o] = na;
+    Key kth = kPad;   // the K1-th approximate distance (warp 0)
+    if (warp == 0) {
+#pragma unroll
+        for (int h = 0; h < NL; ++h) {
+            s_keys[0][lane + 32 * h] = A[h];
+            if (h == (f.K1 - 1) >> 5) kth = A[h];
+        }
+        kth = __shfl_sync(0xffffffffu, kth, (f.K1 - 1) & 31);
+        if (lane == 0) s_na[0] = na;
+    }
+    __syncthreads();
+    const int m = s_na[0];
+    const float *qq = f.Q + q * (int64_t)f.d;
+    // exact distances: lane j of a warp sums the dimensions j, j + 32, ...,
+    // the lanes' sums by a shuffle tree
+    for (int e0 = warp * 4; e0 < m; e0 += 4 * WQ) {
+        const float *x[4];
+        float acc[4] = {0.f, 0.f, 0.f, 0.f};
+        uint32_t id[4];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            id[c] = (uint32_t)s_keys[0][min(e0 + c, m - 1)];
+            x[c] = f.X + (int64_t)id[c] * f.d;
+        }
+        if (f.metric == ESG_L2SQ) {
+#pragma unroll 4
+            for (int j = lane; j < f.d; j += 32) {
+                const float qv = qq[j];
+#pragma unroll
+                for (int c = 0; c < 4; ++c) { const float t = qv - x[c][j]; acc[c] = fmaf(t, t, acc[c]); }
+            }
+        } else {
+#pragma unroll 4
+            for (int j = lane; j < f.d; j += 32) {
+                const float qv = qq[j];
+#pragma unroll
+                for (int c = 0; c < 4; ++c) acc[c] = fmaf(qv, x[c][j], acc[c]);
+            }
+        }
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            acc[c] = warp_sum_group(acc[c], 32);
+            if (lane == 0 && e0 + c < m)
+                s_keys[1][e0 + c] = make_key(f.metric == ESG_L2SQ ? acc[c] : -acc[c], id[c]);
+        }
+    }
+    __syncthreads();
+    if (warp != 0) return;
+    Key R[NL];
+#pragma unroll
+    for (int h = 0; h < NL; ++h) R[h] = lane + 32 * h < m ? s_keys[1][lane + 32 * h] : kPad;
+    sort_asc<NL>(R, lane);
+    const int c = min(f.k, m);
+    Key last = kPad;
+#pragma unroll
+    for (int h = 0; h < NL; ++h)
+        if (h == (max(c, 1) - 1) >> 5) last = R[h];
+    last = __shfl_sync(0xffffffffu, last, (max(c, 1) - 1) & 31);
+    bool certified = c > 0;
+    if (m == f.K1) {   // the list is full: points may have been left out
+        // |approximate - exact| for any point of the range (unit roundoff of
+        // BF16 2^-8, of FP32 2^-24): the split residuals and the dropped
+        // lo*lo product stay below 3.1 * 2^-16 |q_i||x_i| per term, the FP32
+        // accumulation of 3d products below 6d * 2^-24 (twice the rounding
+        // bound, for truncating adders); the squared distance doubles the dot
+        // product error and adds the rounding of the norms and the final sum.
+        const double qn = f.qrownorm[q], xm = f.xmax[0];
+        const double dot_err = (3.1 * 0x1p-16 + 6.0 * f.d * 0x1p-24) * qn * xm;
+        const bool l2 = f.metric == ESG_L2SQ;
+        const double delta = l2 ? 2.0 * dot_err + (f.d + 4.0) * 0x1p-24 * (qn * qn + xm * xm) : dot_err;
+        // list distances leave out the query's squared norm
+        const double bound = (double)key_dist(kth) + (l2 ? (double)f.qnorm[q] : 0.0) - delta;
+        // the re-ranked FP32 distance itself is within d * 2^-23 relative
+        const double dk = (double)key_dist(last);
+        certified = dk + fabs(dk) * f.d * 0x1p-23 < bound;
+    }
+#pragma unroll
+    for (int h = 0; h < NL; ++h) {
+        const int e = lane + 32 * h;
+        if (e < f.k) {
+            f.out_ids[q * f.k + e] = e < c ? (int64_t)(uint32_t)R[h] : -1;
+            f.out_dist[q * f.k + e] = e < c ? key_dist(R[h]) : INFINITY;
+        }
+    }
+    if (lane == 0) { f.out_count[q] = c; f.redo[q] = certified ? 0 : 1; }
+}
+
+// Queries with an invalid range (in no query tile): no results.
+__global__ void invalid_kernel(const int64_t *l, const int64_t *r, int64_t nq, int64_t n, int k, int64_t *out_ids,
+                               float *out_dist, int32_t *out_count, int32_t *redo) {
+    const int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (q >= nq || (l[q] >= 0 && l[q] <= r[q] && r[q] < n)) return;
+    for (int j = 0; j < k; ++j) { out_ids[q * k + j] = -1; out_dist[q * k + j] = INFINITY; }
+    out_count[q] = 0;
+    redo[q] = 0;
 }
 
 }  // namespace
 
-// Exact FP32 re-rank of the candidate lists and certificate. The queries left
-// uncertified go to `leftover` when it is given, else through the exact SIMT
-// pass here.
-static esg_status certify_and_redo(const float *base, int64_t n, int32_t d, int metric, const float *queries,
-                                   int64_t nq, const int64_t *l, const int64_t *r, int32_t k, int K1,
-                                   const float *cand_d, const int32_t *cand_i, const int32_t *cand_n,
-                                   const float *qrow, const float *xmax, int32_t *redo, const int32_t *err,
-                                   int64_t *out_ids, float *out_dist, int32_t *out_count, cudaStream_t stream,
-                                   std::vector<int64_t> *leftover = nullptr) {
-    rerank_certify_kernel<<<ceil_div_i(nq, 4), 128, 0, stream>>>(
-        base, queries, d, metric, nq, k, K1, cand_d, cand_i, cand_n, qrow, xmax, out_ids, out_dist, out_count, redo);
-    cudaError_t ce = cudaGetLastError();
-    if (ce != cudaSuccess) { esg_set_error(cudaGetErrorString(ce)); return ESG_ERR_CUDA; }
+// Waits for the pass and returns the queries it left uncertified.
+static esg_status read_uncertified(int64_t nq, int K1, const int32_t *redo, const int32_t *err, cudaStream_t stream,
+                                   std::vector<int64_t> &idx) {
     std::vector<int32_t> h_redo(nq);
     int32_t h_err = 0;
-    ce = cudaMemcpyAsync(h_redo.data(), redo, sizeof(int32_t) * nq, cudaMemcpyDeviceToHost, stream);
+    cudaError_t ce = cudaMemcpyAsync(h_redo.data(), redo, sizeof(int32_t) * nq, cudaMemcpyDeviceToHost, stream);
     if (ce == cudaSuccess) ce = cudaMemcpyAsync(&h_err, err, sizeof(int32_t), cudaMemcpyDeviceToHost, stream);
     if (ce == cudaSuccess) ce = cudaStreamSynchronize(stream);
     if (ce != cudaSuccess) { esg_set_error(cudaGetErrorString(ce)); return ESG_ERR_CUDA; }
     if (h_err) { esg_set_error("tensor-core brute force: an mbarrier wait timed out"); return ESG_ERR_TIMEOUT; }
-    std::vector<int64_t> idx;
+    idx.clear();
     for (int64_t i = 0; i < nq; ++i) if (h_redo[i]) idx.push_back(i);
     const char *dbg = getenv("ESG_BF_STATS");
     if (dbg && *dbg == '1')
         fprintf(stderr, "tensor-core brute force: %lld of %lld queries left uncertified (list of %d)\n",
                 (long long)idx.size(), (long long)nq, K1);
-    if (leftover) { leftover->swap(idx); return ESG_OK; }
-    if (idx.empty()) return ESG_OK;
-    return esg_bruteforce_redo(base, n, d, metric, queries, nq, l, r, k, idx, out_ids, out_dist, out_count, stream);
+    return ESG_OK;
 }
 
-// Shared-memory plan of the pipelined kernel for a dimension and list length:
-// the query tile resident when that leaves room for two point stages, else
-// streamed with the point chunks (stages of 64 KB); ESG_ERR_UNSUPPORTED when
-// not even two streamed stages fit.
-static esg_status bf2_smem(int32_t d, int K1, int max_smem, int *S, size_t *smem, int *stream_a) {
+// Length of the register lists that serve lists of K1, 0 if they are too long.
+static int bf2_reg_list(int K1) { return K1 == 24 || K1 == 32 ? K1 : 0; }
+
+// Launch plan of the pipelined kernel: query tile in tensor memory (d <= 256),
+// with as many accumulators as fit beside it, or streamed with the point
+// chunks; stages that fit shared memory. ESG_ERR_UNSUPPORTED when not even two
+// stages fit.
+static esg_status bf2_smem(int32_t d, int K1, int max_smem, int *S, size_t *smem, int *n_acc, bool *stream_a,
+                           bool *list_smem) {
     if (K1 > kMaxK1v2 || d < 1) return ESG_ERR_UNSUPPORTED;
     const int nk = (d + TK - 1) / TK;
-    const size_t common = 1024 + (size_t)TM * kTS * 4 + 8 * TN * 4 + (size_t)TM * K1 * 8 + 6 * TM * 4 + 8 * 4 +
-                          8 * (2 * kMaxStages + 8) + 16;
-    const size_t resident = common + (size_t)nk * STAGE;
-    if ((size_t)max_smem >= resident + 2 * (size_t)STAGE) {
-        *stream_a = 0;
-        *S = (int)std::min<size_t>(kMaxStages, ((size_t)max_smem - resident) / STAGE);
-        *smem = resident + (size_t)*S * STAGE;
-        return ESG_OK;
-    }
-    if ((size_t)max_smem < common + 4 * (size_t)STAGE) return ESG_ERR_UNSUPPORTED;
-    *stream_a = 1;
-    *S = (int)std::min<size_t>(kMaxStages, ((size_t)max_smem - common) / (2 * STAGE));
-    *smem = common + (size_t)*S * 2 * STAGE;
+    *stream_a = nk > kMaxResident;
+    *n_acc = *stream_a ? 4 : std::min(3, (kTmem - 64 * nk) / TN);
+    const size_t stage = *stream_a ? 2 * (size_t)STAGE : (size_t)STAGE;
+    // pending slots, tile norms, published distances, mbarriers
+    const bool reg = bf2_reg_list(K1) > 0;
+    const int pend = reg ? 16 : (*stream_a ? Epi<true>::kPend : Epi<false>::kPend);
+    size_t common = sizeof(float2) * kEpiWarps * pend * (reg ? 32 : kPendStride) + sizeof(float) * kEpiWarps * TN +
+                    sizeof(Key) * 4 * TM + 8 * (2 * kMaxStages + 16) + 16;
+    if ((size_t)max_smem < common + 2 * stage) return ESG_ERR_UNSUPPORTED;
+    // the lists in shared memory where they leave four stages (a list in
+    // global memory is a trip to the L2, busy with operand blocks, per merge)
+    const size_t lists = sizeof(Key) * 2 * TM * K1;
+    *list_smem = !reg && (size_t)max_smem >= common + lists + 4 * stage;
+    if (*list_smem) common += lists;
+    *S = (int)std::min<size_t>(kMaxStages, ((size_t)max_smem - common) / stage);
+    *smem = common + (size_t)*S * stage;
     return ESG_OK;
 }
 
@@ -949,13 +1270,7 @@ static esg_status bf2_escalate(const PreparedX &X, const float *base, int64_t n,
                                const float *queries, int64_t nq, const int64_t *l, const int64_t *r, int32_t k,
                                int K1, const std::vector<int64_t> &idx, int64_t *out_ids, float *out_dist,
                                int32_t *out_count, cudaStream_t stream) {
-    int dev = 0, max_smem = 0, S = 0;
-    size_t smem = 0;
-    ESG_CUDA_TRY(cudaGetDevice(&dev));
-    ESG_CUDA_TRY(cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-    int K2 = kMaxK1v2;   // the longest list that fits
-    int sa_mode = 0;
-    while (K2 > K1 && bf2_smem(d, K2, max_smem, &S, &smem, &sa_mode) != ESG_OK) --K2;
+    const int K2 = (d + TK - 1) / TK == 1 ? kMaxK1v2 : kMaxK1v2 - 6;
     if (K2 <= K1)
         return esg_bruteforce_redo(base, n, d, metric, queries, nq, l, r, k, idx, out_ids, out_dist, out_count, stream);
     const int64_t m = (int64_t)idx.size();
@@ -996,28 +1311,42 @@ static esg_status bf2_escalate(const PreparedX &X, const float *base, int64_t n,
 // prepared points, then merge, re-rank, certificate and escalation.
 // Cuts the sequence of covered point tiles (query tile by query tile) into G
 // contiguous shares of about equal estimated cost. A share's cost is its
-// number of tiles plus `restart` for every (query, work item) pair in which
-// the query covers at least one of the item's tiles: a row list starts empty
-// at each item, and while it fills the epilogue inserts many candidates per
-// tile. Per-CTA clock counters at d = 128 (two 64-wide K chunks) put a list
-// start at about six tiles of MMA and filter time (the later insertions did
-// not improve the fit). The epilogue work does not grow with d while a tile's
-// MMA work does, and the longer MMA time per tile also hides more of the
-// burst: the weight 6.25 (2 / nk)^2 tiles fits the best measured weights at
-// d = 128 (6.25) and d = 768 (0 to 0.5, where equal shares are as good).
-// Each cut inside a query tile costs the restarts of the lists of the queries
-// that span it. The shares are chosen greedily: each CTA takes about the
-// remaining cost over the remaining CTAs; every later pass adds the restart
-// cost of the previous pass's later cuts to the remaining cost, and the pass
-// with the smallest largest share is kept. `lt`/`rt` are the first and last
-// covered tile of each sorted query; `cut` receives G + 1 positions.
+// number of tiles plus, for every row with a list, a weight for starting it: a
+// list that starts empty takes many insertions while it fills, and a row
+// insertion costs the same whether one row of the warp or all 32 insert. Rows
+// that start with the item (their ranges begin before it) fill their lists
+// together and share that cost, rows whose ranges begin inside it hardly do;
+// a dense row costs a little for each of its tiles (its stores). The shares
+// are chosen greedily: each CTA takes about the remaining cost over the
+// remaining CTAs; a later pass (of the inspected plan) adds the restart cost of
+// the previous pass's later cuts to the remaining cost, and the pass with the
+// smallest largest share is kept. `lt`/`rt` are the first and last covered
+// tile of each sorted query; `cut` receives G + 1 positions.
 constexpr double kRestart2 = 6.25;   // one list start, in tiles, at two K chunks
 constexpr int kSharePasses = 2;      // greedy passes (the first without restart look-ahead)
 
-static void bf2_shares(const std::vector<int32_t> &tiles, const std::vector<int64_t> &qt_first,
-                       const std::vector<int32_t> &lt, const std::vector<int32_t> &rt, int64_t G,
-                       double restart, std::vector<int64_t> &cut) {
-    const int64_t T = (int64_t)tiles.size(), nqt = (int64_t)qt_first.size() - 1;
+// In tiles: a row whose range begins inside the item, one that begins before
+// it (its list starts with the item, along with the other rows' lists), and a
+// tile of a dense row.
+struct ShareCost {
+    double begin, restart, dense;
+};
+
+// The covered tiles of the query tiles as spans [a, b] of consecutive tiles.
+struct Spans {
+    std::vector<int32_t> a, b, first;   // first: [nqt + 1] first span of each query tile
+    std::vector<int64_t> at;            // position of each span's first tile in the sequence
+    int32_t tile(int64_t qt, int64_t pos) const {
+        int32_t i = first[qt + 1] - 1;
+        while (at[i] > pos) --i;
+        return a[i] + (int32_t)(pos - at[i]);
+    }
+};
+
+static void bf2_shares(const Spans &sp, const std::vector<int64_t> &qt_first, const std::vector<int32_t> &lt,
+                       const std::vector<int32_t> &rt, const std::vector<int32_t> &dense, int64_t G,
+                       const ShareCost &w, int passes, std::vector<int64_t> &cut) {
+    const int64_t nqt = (int64_t)qt_first.size() - 1, T = qt_first[nqt];
     const int64_t nv = (int64_t)lt.size();
     cut.assign(G + 1, T);
     cut[0] = 0;
@@ -1025,12 +1354,18 @@ static void bf2_shares(const std::vector<int32_t> &tiles, const std::vector<int6
     // estimated cost of tiles [t0, t1) of query tile qt, run as one item
     auto cost = [&](int64_t qt, int64_t t0, int64_t t1) -> double {
         if (t1 <= t0) return 0.0;
-        const int32_t a = tiles[t0], b = tiles[t1 - 1];
-        const int32_t *lq = lt.data() + qt * TM, *rq = rt.data() + qt * TM;
+        const int32_t a = sp.tile(qt, t0), b = sp.tile(qt, t1 - 1);
+        const int32_t *lq = lt.data() + qt * TM, *rq = rt.data() + qt * TM, *dq = dense.data() + qt * TM;
         const int ns = (int)(std::min(nv, (qt + 1) * TM) - qt * TM);
-        int nover = 0;
-        for (int s = 0; s < ns; ++s) nover += rq[s] >= a && lq[s] <= b;
-        return (double)(t1 - t0) + restart * nover;
+        int32_t begin = 0, over = 0, dtiles = 0;
+        for (int s = 0; s < ns; ++s) {   // no branches: it vectorises
+            const int32_t l = std::max(lq[s], a), r = std::min(rq[s], b);
+            const int32_t in = l <= r ? 1 : 0;
+            dtiles += dq[s] & ((r - l + 1) * in);
+            over += ~dq[s] & in;
+            begin += ~dq[s] & in & (lq[s] > a ? 1 : 0);
+        }
+        return (double)(t1 - t0) + w.restart * (over - begin) + w.begin * begin + w.dense * dtiles;
     };
     std::vector<double> pre(nqt + 1, 0.0);   // prefix sums of whole query tiles
     for (int64_t qt = 0; qt < nqt; ++qt) pre[qt + 1] = pre[qt] + cost(qt, qt_first[qt], qt_first[qt + 1]);
@@ -1099,7 +1434,7 @@ static void bf2_shares(const std::vector<int32_t> &tiles, const std::vector<int6
     std::vector<int64_t> cur, nxt;
     double best = greedy(later, cur);
     cut = cur;
-    for (int pass = 1; pass < kSharePasses; ++pass) {
+    for (int pass = 1; pass < passes; ++pass) {
         // restart cost of each cut of the previous pass (the next share's head
         // plus the query tile's cost up to the cut, minus the whole query
         // tile), summed over the later cuts
@@ -1126,59 +1461,105 @@ static void bf2_shares(const std::vector<int32_t> &tiles, const std::vector<int6
 // items at query-tile boundaries. ESG_ERR_UNSUPPORTED past 2^31 covered tiles.
 struct Bf2Plan {
     std::vector<int32_t> order;        // sorted position -> caller's query index (valid queries)
-    std::vector<int32_t> tiles;        // covered point tiles, query tile by query tile
+    Spans spans;                       // covered point tiles of each query tile
     std::vector<int64_t> qt_first;     // [nqt + 1] first position of each query tile in `tiles`
     std::vector<WorkItem> items;       // in query-tile order, each CTA's items contiguous
     std::vector<int32_t> item_begin;   // [nqt + 1] first item of each query tile
     std::vector<int32_t> cta_first;    // [G + 1] first item of each CTA
-    int64_t nv = 0, nqt = 0, total_tiles = 0, G = 0, largest = 0;
+    std::vector<int64_t> doff;         // [V] first entry of a dense row in its buffer, -1 for the others
+    int64_t nv = 0, nqt = 0, total_tiles = 0, G = 0, largest = 0, dense = 0;   // dense: floats of all dense rows
 };
 
-static esg_status bf2_plan(const int64_t *hl, const int64_t *hr, int64_t nq, int64_t n, int32_t d, int64_t sms,
-                           Bf2Plan &P) {
-    // sort key floor(log2 width) << 40 | l (l < 2^31), ties by query index:
-    // a stable LSD radix sort by bytes of the key over the valid queries in
-    // index order
-    struct Key { uint64_t k; int32_t i; };
-    std::vector<Key> keys, tmp;
-    keys.reserve(nq);
-    uint64_t kmax = 0;
-    for (int64_t i = 0; i < nq; ++i)
-        if (hl[i] >= 0 && hl[i] <= hr[i] && hr[i] < n) {
-            const uint64_t wb = 63 - __builtin_clzll((unsigned long long)(hr[i] - hl[i] + 1));
-            keys.push_back(Key{(wb << 40) | (uint64_t)hl[i], (int32_t)i});
-            kmax = std::max(kmax, keys.back().k);
+// Rows of narrow ranges write all their distances (the finish kernel selects
+// from them) instead of keeping lists. Ranges that begin inside a work item
+// start their lists one row at a time, and a list start costs a CTA about
+// 27,000 cycles of insertions, one row of the warp active in each; a dense row
+// costs it about 25 cycles per tile (its 16-byte stores). The lines cross at
+// about 135,000 points at d <= 128. At larger d, where a tile's MMAs take longer
+// and hide the insertions, dense rows only add memory traffic (1.66 against 1.50
+// ms at 200,003 x 768). The buffer's bound halves the width until it fits.
+constexpr int64_t kDenseWidth = 131072;
+constexpr int64_t kDenseFloats = (int64_t)1 << 28;   // 1 GiB at most
+
+static void bf2_dense(const int64_t *hl, const int64_t *hr, int64_t widest, Bf2Plan &P) {
+    P.doff.assign(P.order.size(), -1);
+    for (int64_t w = widest; w >= 64; w /= 2) {
+        P.dense = 0;
+        for (size_t s = 0; s < P.order.size(); ++s) {
+            const int64_t l = hl[P.order[s]], r = hr[P.order[s]];
+            const bool in = r - l + 1 <= w;
+            P.doff[s] = in ? P.dense : -1;
+            if (in) P.dense += (r | 3) - (l & ~(int64_t)3) + 1;
         }
-    tmp.resize(keys.size());
-    for (int sh = 0; sh < 64 && (kmax >> sh) != 0; sh += 8) {
-        size_t cnt[257] = {0};
-        for (const Key &x : keys) ++cnt[((x.k >> sh) & 255) + 1];
-        for (int b = 0; b < 256; ++b) cnt[b + 1] += cnt[b];
-        for (const Key &x : keys) tmp[cnt[(x.k >> sh) & 255]++] = x;
+        if (P.dense <= kDenseFloats) return;
+    }
+    P.dense = 0;
+    std::fill(P.doff.begin(), P.doff.end(), (int64_t)-1);
+}
+
+// `run`: the plan is for the kernel (dense rows, its restart cost), not for
+// inspection.
+static esg_status bf2_plan(const int64_t *hl, const int64_t *hr, int64_t nq, int64_t n, int32_t d, int64_t sms,
+                           bool run, Bf2Plan &P) {
+    // sorted by (floor(log2 width), l, query index): a stable LSD radix sort
+    // of the valid queries in index order, by 11 bits of l at a time and then
+    // by the width class
+    std::vector<uint64_t> keys, tmp;   // l << 32 | query
+    keys.reserve(nq);
+    for (int64_t i = 0; i < nq; ++i)
+        if (hl[i] >= 0 && hl[i] <= hr[i] && hr[i] < n) keys.push_back((uint64_t)hl[i] << 32 | (uint32_t)i);
+    const int64_t nv = (int64_t)keys.size();
+    const int64_t nqt = (nv + TM - 1) / TM;
+    const int nk = (d + TK - 1) / TK;
+    tmp.resize(nv);
+    std::vector<uint32_t> cnt(2049);
+    for (int sh = 32; (uint64_t)(n - 1) >> (sh - 32) != 0 && sh < 63; sh += 11) {
+        std::fill(cnt.begin(), cnt.end(), 0u);
+        for (const uint64_t k : keys) ++cnt[((k >> sh) & 2047) + 1];
+        for (int b = 0; b < 2048; ++b) cnt[b + 1] += cnt[b];
+        for (const uint64_t k : keys) tmp[cnt[(k >> sh) & 2047]++] = k;
         keys.swap(tmp);
     }
     std::vector<int32_t> &order = P.order;
-    order.resize(keys.size());
-    for (size_t s = 0; s < keys.size(); ++s) order[s] = keys[s].i;
-    const int64_t nv = (int64_t)order.size();
-    const int64_t nqt = (nv + TM - 1) / TM;
-    const int nk = (d + TK - 1) / TK;
-    std::vector<std::vector<std::pair<int64_t, int64_t>>> spans(nqt);
+    order.resize(nv);
+    {
+        auto cls = [&](uint64_t k) {
+            const int64_t i = (int64_t)(k & 0xFFFFFFFFu);
+            return 63 - __builtin_clzll((unsigned long long)(hr[i] - hl[i] + 1));
+        };
+        uint32_t c[65] = {0};
+        for (const uint64_t k : keys) ++c[cls(k) + 1];
+        for (int b = 0; b < 64; ++b) c[b + 1] += c[b];
+        for (const uint64_t k : keys) order[c[cls(k)]++] = (int32_t)(k & 0xFFFFFFFFu);
+    }
+    // covered tiles of each query tile, as spans
+    Spans &sp = P.spans;
+    sp.first.assign(nqt + 1, 0);
+    std::vector<int64_t> &qt_first = P.qt_first;
+    qt_first.assign(nqt + 1, 0);
     int64_t total_tiles = 0;
-    std::vector<std::pair<int64_t, int64_t>> iv;
-    iv.reserve(TM);
-    for (int64_t qt = 0; qt < nqt; ++qt) {
-        iv.clear();
-        for (int64_t s = qt * TM; s < std::min(nv, (qt + 1) * TM); ++s)
-            iv.push_back({hl[order[s]] / TN, hr[order[s]] / TN});
-        if (!std::is_sorted(iv.begin(), iv.end())) std::sort(iv.begin(), iv.end());
-        for (auto &x : iv) {
-            if (!spans[qt].empty() && x.first <= spans[qt].back().second + 1)
-                spans[qt].back().second = std::max(spans[qt].back().second, x.second);
-            else
-                spans[qt].push_back(x);
+    {
+        std::vector<std::pair<int32_t, int32_t>> iv(TM);
+        for (int64_t qt = 0; qt < nqt; ++qt) {
+            const int64_t s0 = qt * TM, s1 = std::min(nv, (qt + 1) * TM);
+            for (int64_t s = s0; s < s1; ++s)
+                iv[s - s0] = {(int32_t)(hl[order[s]] / TN), (int32_t)(hr[order[s]] / TN)};
+            if (!std::is_sorted(iv.begin(), iv.begin() + (s1 - s0))) std::sort(iv.begin(), iv.begin() + (s1 - s0));
+            for (int64_t s = 0; s < s1 - s0; ++s) {
+                if ((int64_t)sp.a.size() > sp.first[qt] && iv[s].first <= sp.b.back() + 1) {
+                    sp.b.back() = std::max(sp.b.back(), iv[s].second);
+                } else {
+                    sp.a.push_back(iv[s].first);
+                    sp.b.push_back(iv[s].second);
+                }
+            }
+            for (size_t x = sp.first[qt]; x < sp.a.size(); ++x) {
+                sp.at.push_back(total_tiles);
+                total_tiles += sp.b[x] - sp.a[x] + 1;
+            }
+            sp.first[qt + 1] = (int32_t)sp.a.size();
+            qt_first[qt + 1] = total_tiles;
         }
-        for (auto &x : spans[qt]) total_tiles += x.second - x.first + 1;
     }
     // the rows of each full query tile interleaved over the four TMEM lane
     // quarters (sorted position s -> row (s mod 4) * 32 + s / 4): queries
@@ -1194,23 +1575,24 @@ static esg_status bf2_plan(const int64_t *hl, const int64_t *hr, int64_t nq, int
     // tile); CTA c runs the share [cut[c], cut[c + 1]) of it, shares of equal
     // estimated cost, cut into work items at query-tile boundaries (items in
     // query-tile order, each CTA's items contiguous)
-    std::vector<int32_t> &tiles = P.tiles;
-    tiles.resize(total_tiles);
-    std::vector<int64_t> &qt_first = P.qt_first;
-    qt_first.assign(nqt + 1, 0);
-    int64_t pos = 0;
-    for (int64_t qt = 0; qt < nqt; ++qt) {
-        qt_first[qt] = pos;
-        for (auto &x : spans[qt])
-            for (int64_t t = x.first; t <= x.second; ++t) tiles[pos++] = (int32_t)t;
-    }
-    qt_first[nqt] = pos;
     const int64_t G = std::max<int64_t>(1, std::min<int64_t>(sms, total_tiles));
     std::vector<int64_t> cut;
     {
-        std::vector<int32_t> lt(nv), rt(nv);
-        for (int64_t s = 0; s < nv; ++s) { lt[s] = (int32_t)(hl[order[s]] / TN); rt[s] = (int32_t)(hr[order[s]] / TN); }
-        bf2_shares(tiles, qt_first, lt, rt, G, kRestart2 * (2.0 / nk) * (2.0 / nk), cut);
+        std::vector<int32_t> lt(nv), rt(nv), dense(nv, 0);
+        if (run) bf2_dense(hl, hr, nk <= 2 ? kDenseWidth : 0, P);
+        for (int64_t s = 0; s < nv; ++s) {
+            lt[s] = (int32_t)(hl[order[s]] / TN);
+            rt[s] = (int32_t)(hr[order[s]] / TN);
+            dense[s] = run && P.doff[s] >= 0 ? -1 : 0;
+        }
+        // weights in tiles at two K chunks, from the CTAs' clock counters at
+        // 1M x 128 (27,000 cycles for a row that begins inside the item, 25 for
+        // a dense row's tile, 2,300 for a tile); a tile's MMAs grow with nk,
+        // and past two chunks they hide more and more of the epilogue
+        const double f = 2.0 / nk, g = nk <= 2 ? f : f * f * f;
+        const ShareCost w = run ? ShareCost{16.0 * g, 0.5 * g, 0.0104 * g}
+                                : ShareCost{kRestart2 * f * f, kRestart2 * f * f, 0.0};
+        bf2_shares(sp, qt_first, lt, rt, dense, G, w, run ? 1 : kSharePasses, cut);
     }
     std::vector<WorkItem> &items = P.items;
     items.clear();
@@ -1243,6 +1625,35 @@ static esg_status bf2_plan(const int64_t *hl, const int64_t *hr, int64_t nq, int
     return ESG_OK;
 }
 
+// Writes out the covered tiles of the work items (a block each) from the query
+// tiles' spans. Inside an item the tiles are rotated to begin at the first one
+// at or after a multiple of `period`, about the length of the long items: the
+// CTAs that sweep the same points with different query tiles then read the same
+// blocks at about the same time, and the operand blocks come from DRAM once
+// instead of once per query tile (DRAM reads 10.7 -> 5.7 GB at 1M x
+// 128, 5.5 -> 2.2 GB at 200,003 x 768, whose call takes 1.54 ms instead of 1.65).
+__global__ void expand_tiles_kernel(const WorkItem *items, const int32_t *span_a, const int32_t *span_first,
+                                    const int64_t *span_at, int period, int32_t *tiles) {
+    const WorkItem w = items[blockIdx.x];
+    const int32_t x0 = span_first[w.qtile], x1 = span_first[w.qtile + 1];
+    auto tile = [&](int64_t pos) {
+        int32_t x = x1 - 1;
+        while (x > x0 && span_at[x] > pos) --x;
+        return span_a[x] + (int32_t)(pos - span_at[x]);
+    };
+    // the first tile of the item at or after a multiple of the period
+    const int32_t first = tile(w.off), from = (first + period - 1) / period * period;
+    int lo = 0, hi = w.cnt;
+    while (lo < hi) {
+        const int m = (lo + hi) >> 1;
+        if (tile(w.off + m) < from) lo = m + 1; else hi = m;
+    }
+    for (int j = threadIdx.x; j < w.cnt; j += blockDim.x) {
+        const int k = lo + j < w.cnt ? lo + j : lo + j - w.cnt;
+        tiles[w.off + j] = tile((int64_t)w.off + k);
+    }
+}
+
 // `given`: a plan already made for these ranges (it is consumed), or null.
 static esg_status bf2_queries(const PreparedX &X, const float *base, int64_t n, int32_t d, int metric,
                               const float *queries, int64_t nq, const int64_t *l, const int64_t *r, int32_t k,
@@ -1251,12 +1662,13 @@ static esg_status bf2_queries(const PreparedX &X, const float *base, int64_t n, 
     if (nq == 0) return ESG_OK;
     const double h0 = bf_stats() ? bf_host_ms() : 0.0;
     const int nk = (d + TK - 1) / TK;
-    int dev = 0, max_smem = 0, sms = 0, S = 0, stream_a = 0;
+    int dev = 0, max_smem = 0, sms = 0, S = 0, n_acc = 0;
+    bool stream_a = false, list_smem = false;
     size_t smem = 0;
     ESG_CUDA_TRY(cudaGetDevice(&dev));
     ESG_CUDA_TRY(cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
     ESG_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    if (bf2_smem(d, K1, max_smem, &S, &smem, &stream_a) != ESG_OK) return ESG_ERR_UNSUPPORTED;
+    if (bf2_smem(d, K1, max_smem, &S, &smem, &n_acc, &stream_a, &list_smem) != ESG_OK) return ESG_ERR_UNSUPPORTED;
 
     // ---- host plan
     Bf2Plan P;
@@ -1267,12 +1679,12 @@ static esg_status bf2_queries(const PreparedX &X, const float *base, int64_t n, 
         ESG_CUDA_TRY(cudaMemcpyAsync(hl.data(), l, sizeof(int64_t) * nq, cudaMemcpyDeviceToHost, stream));
         ESG_CUDA_TRY(cudaMemcpyAsync(hr.data(), r, sizeof(int64_t) * nq, cudaMemcpyDeviceToHost, stream));
         ESG_CUDA_TRY(cudaStreamSynchronize(stream));
-        const esg_status pst = bf2_plan(hl.data(), hr.data(), nq, n, d, sms, P);
+        const esg_status pst = bf2_plan(hl.data(), hr.data(), nq, n, d, sms, true, P);
         if (pst != ESG_OK) return pst;
     }
-    const std::vector<int32_t> &order = P.order, &tiles = P.tiles, &item_begin = P.item_begin,
-                               &cta_first = P.cta_first;
+    const std::vector<int32_t> &order = P.order, &item_begin = P.item_begin, &cta_first = P.cta_first;
     const std::vector<WorkItem> &items = P.items;
+    const int64_t n_spans = (int64_t)P.spans.a.size();
     const int64_t nv = P.nv, nqt = P.nqt, total_tiles = P.total_tiles, G = P.G, CH = P.largest;
     const int64_t n_items = (int64_t)items.size();
 
@@ -1282,9 +1694,10 @@ static esg_status bf2_queries(const PreparedX &X, const float *base, int64_t n, 
     size_t bytes = al((size_t)std::max<int64_t>(nqt, 1) * nk * STAGE) + 2 * al(sizeof(float) * nq) +
                    al(sizeof(int32_t) * std::max<int64_t>(nv, 1)) + al(sizeof(WorkItem) * ni1) +
                    al(sizeof(int32_t) * std::max<int64_t>(total_tiles, 1)) + al(sizeof(int32_t) * (nqt + 1)) +
-                   al(sizeof(int32_t) * (G + 1)) + 2 * al((size_t)4 * ni1 * K1 * TM) + al(sizeof(int32_t) * ni1 * TM) +
-                   al((sizeof(float) + sizeof(int32_t)) * (size_t)nq * K1) + 3 * al(sizeof(int32_t) * nq) +
-                   al(sizeof(int32_t) * 4);
+                   al(sizeof(int32_t) * (G + 1)) + al(sizeof(Key) * 2 * ni1 * K1 * TM) +
+                   al(sizeof(int32_t) * 2 * ni1 * TM) + al(sizeof(int32_t) * nq) + al(sizeof(int32_t) * 4) +
+                   al(sizeof(int64_t) * std::max<int64_t>(nv, 1)) + al(sizeof(float) * P.dense) +
+                   al(sizeof(int32_t) * n_spans) + al(sizeof(int64_t) * n_spans) + al(sizeof(int32_t) * (nqt + 1));
     unsigned char *scratch = nullptr;
     ESG_CUDA_TRY(esg_malloc_async((void **)&scratch, bytes, stream));
     unsigned char *p = scratch;
@@ -1297,24 +1710,41 @@ static esg_status bf2_queries(const PreparedX &X, const float *base, int64_t n, 
     int32_t *d_tiles = (int32_t *)take(sizeof(int32_t) * std::max<int64_t>(total_tiles, 1));
     int32_t *d_ib = (int32_t *)take(sizeof(int32_t) * (nqt + 1));
     int32_t *d_cta = (int32_t *)take(sizeof(int32_t) * (G + 1));
-    float *part_d = (float *)take((size_t)4 * ni1 * K1 * TM);
-    int32_t *part_i = (int32_t *)take((size_t)4 * ni1 * K1 * TM);
-    int32_t *part_n = (int32_t *)take(sizeof(int32_t) * ni1 * TM);
-    float *cand_d = (float *)take(sizeof(float) * (size_t)nq * K1);
-    int32_t *cand_i = (int32_t *)take(sizeof(int32_t) * (size_t)nq * K1);
-    int32_t *cand_n = (int32_t *)take(sizeof(int32_t) * nq);
+    Key *part = (Key *)take(sizeof(Key) * 2 * ni1 * K1 * TM);
+    int32_t *part_n = (int32_t *)take(sizeof(int32_t) * 2 * ni1 * TM);
     int32_t *redo = (int32_t *)take(sizeof(int32_t) * nq);
     int32_t *err = (int32_t *)take(sizeof(int32_t) * 4);
+    int64_t *d_doff = (int64_t *)take(sizeof(int64_t) * std::max<int64_t>(nv, 1));
+    float *dense = (float *)take(sizeof(float) * P.dense);
+    int32_t *d_span_a = (int32_t *)take(sizeof(int32_t) * n_spans);
+    int64_t *d_span_at = (int64_t *)take(sizeof(int64_t) * n_spans);
+    int32_t *d_span_first = (int32_t *)take(sizeof(int32_t) * (nqt + 1));
 
     esg_status st = ESG_OK;
     cudaError_t ce = cudaMemsetAsync(err, 0, sizeof(int32_t) * 4, stream);
-    if (ce == cudaSuccess) ce = cudaMemsetAsync(cand_n, 0xFF, sizeof(int32_t) * nq, stream);   // -1: invalid
     if (ce == cudaSuccess && nv > 0)
         ce = cudaMemcpyAsync(d_order, order.data(), sizeof(int32_t) * nv, cudaMemcpyHostToDevice, stream);
+    if (ce == cudaSuccess && nv > 0)
+        ce = cudaMemcpyAsync(d_doff, P.doff.data(), sizeof(int64_t) * nv, cudaMemcpyHostToDevice, stream);
     if (ce == cudaSuccess && n_items > 0)
         ce = cudaMemcpyAsync(d_items, items.data(), sizeof(WorkItem) * n_items, cudaMemcpyHostToDevice, stream);
-    if (ce == cudaSuccess && total_tiles > 0)
-        ce = cudaMemcpyAsync(d_tiles, tiles.data(), sizeof(int32_t) * total_tiles, cudaMemcpyHostToDevice, stream);
+    if (ce == cudaSuccess && n_items > 0) {
+        ce = cudaMemcpyAsync(d_span_a, P.spans.a.data(), sizeof(int32_t) * n_spans, cudaMemcpyHostToDevice, stream);
+        if (ce == cudaSuccess)
+            ce = cudaMemcpyAsync(d_span_at, P.spans.at.data(), sizeof(int64_t) * n_spans, cudaMemcpyHostToDevice, stream);
+        if (ce == cudaSuccess)
+            ce = cudaMemcpyAsync(d_span_first, P.spans.first.data(), sizeof(int32_t) * (nqt + 1),
+                                 cudaMemcpyHostToDevice, stream);
+        if (ce == cudaSuccess) {
+            std::vector<int32_t> c(n_items);
+            for (int64_t i = 0; i < n_items; ++i) c[i] = items[i].cnt;
+            std::nth_element(c.begin(), c.begin() + n_items * 3 / 4, c.end());
+            const int period = c[n_items * 3 / 4];
+            expand_tiles_kernel<<<(unsigned)n_items, 256, 0, stream>>>(d_items, d_span_a, d_span_first, d_span_at,
+                                                                       period, d_tiles);
+            ce = cudaGetLastError();
+        }
+    }
     if (ce == cudaSuccess)
         ce = cudaMemcpyAsync(d_ib, item_begin.data(), sizeof(int32_t) * (nqt + 1), cudaMemcpyHostToDevice, stream);
     if (ce == cudaSuccess)
@@ -1323,7 +1753,22 @@ static esg_status bf2_queries(const PreparedX &X, const float *base, int64_t n, 
         if (nqt > 0)
             ce = split_norm(queries, nv, d, nk, d_order, nqt * TM, qs, qnorm, qrow, nullptr, stream);
     }
-    if (ce == cudaSuccess) ce = cudaFuncSetAttribute(tc_knn2_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    // lists in 32 or 64 registers-times-lanes
+    const bool l2 = metric == ESG_L2SQ, one = K1 <= 32;
+    auto pick = [&](auto s) -> void (*)(Tc2Args) {
+        constexpr bool ST = decltype(s)::value;
+        switch (bf2_reg_list(K1)) {
+            case 24: return l2 ? tc_knn2_kernel<true, 24, 1, ST> : tc_knn2_kernel<false, 24, 1, ST>;
+            case 32: return l2 ? tc_knn2_kernel<true, 32, 1, ST> : tc_knn2_kernel<false, 32, 1, ST>;
+        }
+        return l2 ? tc_knn2_kernel<true, 0, 2, ST> : tc_knn2_kernel<false, 0, 2, ST>;
+    };
+    void (*fn)(Tc2Args) = stream_a ? pick(std::true_type{}) : pick(std::false_type{});
+    if (ce == cudaSuccess) ce = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (ce == cudaSuccess && nv < nq) {
+        invalid_kernel<<<ceil_div_i(nq, 256), 256, 0, stream>>>(l, r, nq, n, k, out_ids, out_dist, out_count, redo);
+        ce = cudaGetLastError();
+    }
     if (ce == cudaSuccess && n_items > 0) {
         // MMA work issued: three 128 x 128 x 64 BF16 products per point tile and K chunk
         esg_prof_tensor_flops((double)total_tiles * nk * 3.0 * 2.0 * TM * TN * TK);
@@ -1333,15 +1778,28 @@ static esg_status bf2_queries(const PreparedX &X, const float *base, int64_t n, 
         const char *wn = getenv("ESG_BF_WAIT_NS");
         const char *stl = getenv("ESG_TEST_BF_STALL");
         const unsigned long long wait_ns = wn && *wn ? std::max(1ull, strtoull(wn, nullptr, 10)) : kWaitNs;
-        Tc2Args a{X.xs, qs, X.xnorm, qnorm, l, r, d_order, d_items, d_tiles, d_cta, (int)n_items, nv, nk, metric, K1, S,
-                  stream_a, n, part_d, part_i, part_n, err, wait_ns, (stl && atoi(stl) == 1) ? 1 : 0};
+        Tc2Args a{X.xs, qs, X.xnorm, qnorm, l, r, d_order, d_doff, dense, d_items, d_tiles, d_cta, (int)n_items, nv, nk, metric, K1, S,
+                  list_smem ? 1 : 0, n_acc,
+                  // two issuers wait for stages of two tiles: a barrier must
+                  // not be waited for more than one use ahead
+                  !stream_a && 2 * nk <= S ? 2 : 1,
+                  n, part, part_n, err, wait_ns, (stl && atoi(stl) == 1) ? 1 : 0};
         const int pidx = esg_prof_begin(stream);
-        tc_knn2_kernel<<<(unsigned)G, kThreads2, smem, stream>>>(a);
+        fn<<<(unsigned)G, kThreads2, smem, stream>>>(a);
         ce = cudaGetLastError();
         esg_prof_end(pidx, stream);
         if (ce == cudaSuccess) {
-            merge_parts_kernel<<<ceil_div_i(nv, 4), 128, 0, stream>>>(part_d, part_i, part_n, d_ib, d_order, nv, K1,
-                                                                      cand_d, cand_i, cand_n);
+            const FinishArgs f{base, queries, d, metric, k, K1, part, part_n, d_ib, d_order, d_doff, l, r, dense, qnorm, qrow,
+                               X.xmax,
+                               out_ids, out_dist, out_count, redo};
+            // many lists per query: two per item, items shared out over the query tiles
+            if (n_items > 16 * nqt) {
+                if (one) finish_kernel<1, 16><<<(unsigned)nv, 512, 0, stream>>>(f);
+                else finish_kernel<2, 16><<<(unsigned)nv, 512, 0, stream>>>(f);
+            } else {
+                if (one) finish_kernel<1, 4><<<(unsigned)nv, 128, 0, stream>>>(f);
+                else finish_kernel<2, 4><<<(unsigned)nv, 128, 0, stream>>>(f);
+            }
             ce = cudaGetLastError();
         }
     }
@@ -1354,8 +1812,7 @@ static esg_status bf2_queries(const PreparedX &X, const float *base, int64_t n, 
     std::vector<int64_t> left;
     const double h1 = bf_stats() ? bf_host_ms() : 0.0;
     if (st == ESG_OK)
-        st = certify_and_redo(base, n, d, metric, queries, nq, l, r, k, K1, cand_d, cand_i, cand_n, qrow, X.xmax,
-                              redo, err, out_ids, out_dist, out_count, stream, &left);
+        st = read_uncertified(nq, K1, redo, err, stream, left);
     cudaFreeAsync(scratch, stream);
     const double h2 = bf_stats() ? bf_host_ms() : 0.0;
     if (st == ESG_OK && !left.empty())
@@ -1379,18 +1836,15 @@ static esg_status bruteforce_tc_v2(const float *base, int64_t n, int32_t d, int 
     // k + 12 candidates, at least k + 8 (the longest list the kernel holds
     // caps it): at 1M x 128, 10k queries, k = 10, lists of k + 8 left 2 queries
     // uncertified and their second pass cost 0.75 ms of a 5.90 ms call; k + 12
-    // certified all (5.52 ms), k + 16 and k + 24 made the epilogue slower
-    // (5.83, 6.56 ms)
-    if (k < 1 || k + 8 > kMaxK1v2 || n >= ((int64_t)1 << 31) || d < 1) return ESG_ERR_UNSUPPORTED;
-    int K1 = std::min(k + 12, kMaxK1v2);
-    int dev = 0, max_smem = 0, S = 0, stream_a = 0;
+    // certified all
+    if (k < 1 || k + 8 > ((d + TK - 1) / TK == 1 ? kMaxK1v2 : kMaxK1v2 - 6) || n >= ((int64_t)1 << 31) || d < 1) return ESG_ERR_UNSUPPORTED;
+    const int K1 = k <= 12 ? 24 : (k <= 20 ? 32 : std::min(k + 12, kMaxK1v2));
+    int dev = 0, max_smem = 0, S = 0, n_acc = 0;
+    bool stream_a = false, list_smem = false;
     size_t smem = 0;
     ESG_CUDA_TRY(cudaGetDevice(&dev));
     ESG_CUDA_TRY(cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-    if (bf2_smem(d, K1, max_smem, &S, &smem, &stream_a) != ESG_OK) {
-        K1 = k + 8;
-        if (bf2_smem(d, K1, max_smem, &S, &smem, &stream_a) != ESG_OK) return ESG_ERR_UNSUPPORTED;
-    }
+    if (bf2_smem(d, K1, max_smem, &S, &smem, &n_acc, &stream_a, &list_smem) != ESG_OK) return ESG_ERR_UNSUPPORTED;
     if (nq == 0) return ESG_OK;
     const double t0 = bf_stats() ? bf_host_ms() : 0.0;
     const int nk = (d + TK - 1) / TK;
@@ -1404,12 +1858,12 @@ static esg_status bruteforce_tc_v2(const float *base, int64_t n, int32_t d, int 
     ESG_CUDA_TRY(cudaMemcpyAsync(hr.data(), r, sizeof(int64_t) * nq, cudaMemcpyDeviceToHost, stream));
     ESG_CUDA_TRY(cudaStreamSynchronize(stream));
     auto al = [](size_t x) { return (x + 255) & ~(size_t)255; };
-    const size_t bytes = al((size_t)xt * nk * STAGE) + al(sizeof(float) * n) + al(sizeof(float) * 4);
+    const size_t bytes = al((size_t)xt * nk * STAGE) + al(sizeof(float) * xt * TN) + al(sizeof(float) * 4);
     unsigned char *scratch = nullptr;
     ESG_CUDA_TRY(esg_malloc_async((void **)&scratch, bytes, stream));
     unsigned char *p = scratch;
     unsigned char *xs = p; p += al((size_t)xt * nk * STAGE);
-    float *xnorm = (float *)p; p += al(sizeof(float) * n);
+    float *xnorm = (float *)p; p += al(sizeof(float) * xt * TN);   // past n: never in a range
     float *xmax = (float *)p;
     esg_status st = ESG_OK;
     cudaError_t ce = cudaMemsetAsync(xmax, 0, sizeof(float) * 4, stream);
@@ -1419,7 +1873,7 @@ static esg_status bruteforce_tc_v2(const float *base, int64_t n, int32_t d, int 
     if (ce != cudaSuccess) { esg_set_error(cudaGetErrorString(ce)); st = ESG_ERR_CUDA; }
     const double t1 = bf_stats() ? bf_host_ms() : 0.0;
     Bf2Plan P;
-    if (st == ESG_OK) st = bf2_plan(hl.data(), hr.data(), nq, n, d, sms, P);
+    if (st == ESG_OK) st = bf2_plan(hl.data(), hr.data(), nq, n, d, sms, true, P);
     if (bf_stats()) fprintf(stderr, "tensor-core brute force, host ms: ranges + point prep queued %.3f, plan %.3f\n",
                             t1 - t0, bf_host_ms() - t1);
     if (st == ESG_OK) {
@@ -1449,7 +1903,7 @@ esg_status esg_bruteforce_plan(int64_t n, int32_t d, const int64_t *l, const int
     Bf2Plan P;
     esg_status st = ESG_OK;
     try {
-        st = bf2_plan(l, r, nq, n, d, ctas, P);
+        st = bf2_plan(l, r, nq, n, d, ctas, false, P);
     } catch (...) { st = ESG_ERR_OOM; }
     if (st != ESG_OK) {
         if (st == ESG_ERR_UNSUPPORTED) esg_set_error("esg_bruteforce_plan: more than 2^31 covered point tiles");
@@ -1460,7 +1914,9 @@ esg_status esg_bruteforce_plan(int64_t n, int32_t d, const int64_t *l, const int
     sizes[2] = (int64_t)P.items.size();
     sizes[3] = P.G;
     if (order) std::copy(P.order.begin(), P.order.end(), order);
-    if (tiles) std::copy(P.tiles.begin(), P.tiles.end(), tiles);
+    if (tiles)
+        for (size_t x = 0; x < P.spans.a.size(); ++x)
+            for (int32_t t = P.spans.a[x]; t <= P.spans.b[x]; ++t) *tiles++ = t;
     if (items)
         for (size_t i = 0; i < P.items.size(); ++i) {
             items[4 * i] = P.items[i].qtile;

@@ -38,3 +38,52 @@ def test_mlp_batch_edges(B):
     assert abs(loss - ref_loss) <= 1e-5 * max(1.0, abs(ref_loss))
     assert np.max(np.abs(g.cpu().numpy() - ref_g)) <= 1e-4 * np.max(np.abs(ref_g)) + 1e-8
     assert loss == again and torch.equal(g, g2)
+
+
+def _check_exact(X, Q, l, r, k, metric, ids, dist, count):
+    """Exact answers against float64: counts, distances within 1e-5 relative
+    or the forward error bound of the FP32 sum, and every row that float64
+    puts below the k-th distance by more than four times that."""
+    X64, Q64 = torch.as_tensor(X).double(), torch.as_tensor(Q).double()
+    for i in range(len(Q)):
+        a, b = int(l[i]), int(r[i]) + 1
+        terms = (X64[a:b] - Q64[i]) ** 2 if metric == "l2" else -X64[a:b] * Q64[i]
+        d = terms.sum(1)
+        c = min(k, b - a)
+        want, order = torch.sort(d)
+        assert count[i] == c and np.all(ids[i, c:] == -1) and np.all(np.isinf(dist[i, c:]))
+        got = ids[i, :c]
+        assert len(set(got.tolist())) == c and got.min() >= a and got.max() < b
+        bound = X.shape[1] * 2.0 ** -24 * terms.abs().sum(1)
+        tol = np.maximum(1e-5 * np.abs(d.numpy()), bound.numpy())
+        assert np.all(np.abs(dist[i, :c] - d.numpy()[got - a]) <= tol[got - a])
+        assert np.all(np.diff(dist[i, :c]) >= 0)
+        sure = order[:c][want[:c] < want[c - 1] - 4 * tol.max()] + a
+        assert set(sure.tolist()) <= set(got.tolist())
+
+
+@pytest.mark.parametrize("d", [32, 64, 100, 128, 132, 192, 256, 260])
+@pytest.mark.parametrize("metric", ["l2", "ip"])
+@pytest.mark.parametrize("k", [1, 12, 13, 20, 21, 50])
+def test_exact_lists_and_dense_rows(d, metric, k):
+    """Lists of 24 and 32 in registers and of up to 62 in memory, dense rows
+    up to 131,072 points wide and lists above, query tiles in tensor memory
+    (d <= 256, one or two issuers) and streamed; ranges at tile edges, one
+    point, the whole set, and a second, partial query tile."""
+    n, nq = 131_072 + 777, 131
+    g = torch.Generator(device=DEV).manual_seed(d * 100 + k)
+    cen = torch.randn(64, d, generator=g, device=DEV)
+    X = cen[torch.randint(0, 64, (n,), generator=g, device=DEV)] + 0.5 * torch.randn(n, d, generator=g, device=DEV)
+    Q = cen[torch.randint(0, 64, (nq,), generator=g, device=DEV)] + 0.5 * torch.randn(nq, d, generator=g, device=DEV)
+    rng = np.random.default_rng(d + k)
+    w = np.exp(rng.uniform(0, np.log(n), nq)).astype(np.int64)
+    l = (rng.random(nq) * (n - w + 1)).astype(np.int64)
+    r = l + w - 1
+    edge = [(0, n - 1), (0, 131_071), (0, 131_072), (1, n - 1), (0, 0), (n - 1, n - 1), (127, 128), (128, 255),
+            (127, 256), (n - 777, n - 1), (700, 131_771), (500, n - 3)]
+    l[:len(edge)], r[:len(edge)] = zip(*edge)
+    ids, dist, count = E.esg_bruteforce_filtered_knn(X, Q, _t(l), _t(r), k, metric)
+    torch.cuda.synchronize()
+    pick = list(range(len(edge))) + rng.choice(np.arange(len(edge), nq), 12, replace=False).tolist()
+    _check_exact(X.cpu().numpy(), Q.cpu().numpy()[pick], l[pick], r[pick], k, metric, ids.cpu().numpy()[pick],
+                 dist.cpu().numpy()[pick], count.cpu().numpy()[pick])
