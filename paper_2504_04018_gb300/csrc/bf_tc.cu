@@ -248,7 +248,7 @@ constexpr int STAGE = 2 * CHUNK;          // hi + lo of a 128 x 64 block
 constexpr int kEpiWarps = 8;
 constexpr int kMmaWarps = 2;
 constexpr int kThreads2 = 32 + 32 * kMmaWarps + 32 * kEpiWarps;
-constexpr int kMaxK1v2 = 64;              // longest list
+constexpr int kMaxK1v2 = 128;             // longest list
 constexpr int kMaxStages = 6;
 constexpr int kTmem = 512;                // TMEM columns: all, one CTA per SM
 constexpr int kMaxResident = 4;           // 64-wide chunks of a query tile that fit beside two accumulators
@@ -954,6 +954,7 @@ struct FinishArgs {
     const int64_t *doff, *l, *r;
     const float *dense;
     const float *qnorm, *qrownorm, *xmax;
+    int serial;                     // 1: exact distances summed in dimension order
     int64_t *out_ids;
     float *out_dist;
     int32_t *out_count, *redo;
@@ -1084,6 +1085,28 @@ __global__ void __launch_bounds__(32 * WQ) finish_kernel(FinishArgs f) {
     __syncthreads();
     const int m = s_na[0];
     const float *qq = f.Q + q * (int64_t)f.d;
+    if (f.serial) {
+        // one candidate per thread, its terms added in dimension order: what
+        // the SIMT kernel computes, so that answers with these lists do not
+        // depend on which of the two a query went through
+        for (int e = threadIdx.x; e < m; e += 32 * WQ) {
+            const uint32_t id = (uint32_t)s_keys[0][e];
+            const float4 *x4 = (const float4 *)(f.X + (int64_t)id * f.d), *q4 = (const float4 *)qq;
+            float acc = 0.f;
+#pragma unroll 4
+            for (int j = 0; j < f.d / 4; ++j) {
+                const float4 x = __ldg(x4 + j), qv = __ldg(q4 + j);
+                if (f.metric == ESG_L2SQ) {
+                    const float t0 = qv.x - x.x, t1 = qv.y - x.y, t2 = qv.z - x.z, t3 = qv.w - x.w;
+                    acc = fmaf(t0, t0, acc); acc = fmaf(t1, t1, acc); acc = fmaf(t2, t2, acc); acc = fmaf(t3, t3, acc);
+                } else {
+                    acc = fmaf(qv.x, x.x, acc); acc = fmaf(qv.y, x.y, acc);
+                    acc = fmaf(qv.z, x.z, acc); acc = fmaf(qv.w, x.w, acc);
+                }
+            }
+            s_keys[1][e] = make_key(f.metric == ESG_L2SQ ? acc : -acc, id);
+        }
+    } else
     // exact distances: lane j of a warp sums the dimensions j, j + 32, ...,
     // the lanes' sums by a shuffle tree
     for (int e0 = warp * 4; e0 < m; e0 += 4 * WQ) {
@@ -1189,6 +1212,11 @@ static esg_status read_uncertified(int64_t nq, int K1, const int32_t *redo, cons
     return ESG_OK;
 }
 
+// Whether answers for k are summed in dimension order, like the SIMT kernel's
+// (which alone served lists longer than 64, or 58 past 64 dimensions), or over
+// the lanes: a call's rounding stays what it was.
+static bool bf2_serial(int32_t d, int k) { return k + 8 > ((d + TK - 1) / TK == 1 ? 64 : 58); }
+
 // Length of the register lists that serve lists of K1, 0 if they are too long.
 static int bf2_reg_list(int K1) { return K1 == 24 || K1 == 32 ? K1 : 0; }
 
@@ -1270,7 +1298,7 @@ static esg_status bf2_escalate(const PreparedX &X, const float *base, int64_t n,
                                const float *queries, int64_t nq, const int64_t *l, const int64_t *r, int32_t k,
                                int K1, const std::vector<int64_t> &idx, int64_t *out_ids, float *out_dist,
                                int32_t *out_count, cudaStream_t stream) {
-    const int K2 = (d + TK - 1) / TK == 1 ? kMaxK1v2 : kMaxK1v2 - 6;
+    const int K2 = bf2_serial(d, k) ? kMaxK1v2 : ((d + TK - 1) / TK == 1 ? 64 : 58);
     if (K2 <= K1)
         return esg_bruteforce_redo(base, n, d, metric, queries, nq, l, r, k, idx, out_ids, out_dist, out_count, stream);
     const int64_t m = (int64_t)idx.size();
@@ -1478,10 +1506,13 @@ struct Bf2Plan {
 // about 135,000 points at d <= 128. At larger d, where a tile's MMAs take longer
 // and hide the insertions, dense rows only add memory traffic (1.66 against 1.50
 // ms at 200,003 x 768). The buffer's bound halves the width until it fits.
+// Lists in memory cost several times the insertions: rows up to twice as wide
+// are dense, in a buffer twice as large (1M x 96, 10k queries, k = 100: 9.5 ms a
+// call, 179 ms through the SIMT kernel).
 constexpr int64_t kDenseWidth = 131072;
 constexpr int64_t kDenseFloats = (int64_t)1 << 28;   // 1 GiB at most
 
-static void bf2_dense(const int64_t *hl, const int64_t *hr, int64_t widest, Bf2Plan &P) {
+static void bf2_dense(const int64_t *hl, const int64_t *hr, int64_t widest, int64_t most, Bf2Plan &P) {
     P.doff.assign(P.order.size(), -1);
     for (int64_t w = widest; w >= 64; w /= 2) {
         P.dense = 0;
@@ -1491,16 +1522,16 @@ static void bf2_dense(const int64_t *hl, const int64_t *hr, int64_t widest, Bf2P
             P.doff[s] = in ? P.dense : -1;
             if (in) P.dense += (r | 3) - (l & ~(int64_t)3) + 1;
         }
-        if (P.dense <= kDenseFloats) return;
+        if (P.dense <= most) return;
     }
     P.dense = 0;
     std::fill(P.doff.begin(), P.doff.end(), (int64_t)-1);
 }
 
-// `run`: the plan is for the kernel (dense rows, its restart cost), not for
-// inspection.
+// `run`: the plan is for the kernel with lists of K1 (dense rows, its restart
+// cost), not for inspection.
 static esg_status bf2_plan(const int64_t *hl, const int64_t *hr, int64_t nq, int64_t n, int32_t d, int64_t sms,
-                           bool run, Bf2Plan &P) {
+                           bool run, int K1, Bf2Plan &P) {
     // sorted by (floor(log2 width), l, query index): a stable LSD radix sort
     // of the valid queries in index order, by 11 bits of l at a time and then
     // by the width class
@@ -1579,7 +1610,8 @@ static esg_status bf2_plan(const int64_t *hl, const int64_t *hr, int64_t nq, int
     std::vector<int64_t> cut;
     {
         std::vector<int32_t> lt(nv), rt(nv), dense(nv, 0);
-        if (run) bf2_dense(hl, hr, nk <= 2 ? kDenseWidth : 0, P);
+        const int64_t x = K1 > 32 ? 2 : 1;
+        if (run) bf2_dense(hl, hr, nk <= 2 ? x * kDenseWidth : 0, x * kDenseFloats, P);
         for (int64_t s = 0; s < nv; ++s) {
             lt[s] = (int32_t)(hl[order[s]] / TN);
             rt[s] = (int32_t)(hr[order[s]] / TN);
@@ -1590,7 +1622,8 @@ static esg_status bf2_plan(const int64_t *hl, const int64_t *hr, int64_t nq, int
         // a dense row's tile, 2,300 for a tile); a tile's MMAs grow with nk,
         // and past two chunks they hide more and more of the epilogue
         const double f = 2.0 / nk, g = nk <= 2 ? f : f * f * f;
-        const ShareCost w = run ? ShareCost{16.0 * g, 0.5 * g, 0.0104 * g}
+        const double c = K1 > 32 ? K1 / 24.0 : 1.0;   // insertions grow with the list
+        const ShareCost w = run ? ShareCost{16.0 * c * g, 0.5 * c * g, 0.0104 * g}
                                 : ShareCost{kRestart2 * f * f, kRestart2 * f * f, 0.0};
         bf2_shares(sp, qt_first, lt, rt, dense, G, w, run ? 1 : kSharePasses, cut);
     }
@@ -1679,7 +1712,7 @@ static esg_status bf2_queries(const PreparedX &X, const float *base, int64_t n, 
         ESG_CUDA_TRY(cudaMemcpyAsync(hl.data(), l, sizeof(int64_t) * nq, cudaMemcpyDeviceToHost, stream));
         ESG_CUDA_TRY(cudaMemcpyAsync(hr.data(), r, sizeof(int64_t) * nq, cudaMemcpyDeviceToHost, stream));
         ESG_CUDA_TRY(cudaStreamSynchronize(stream));
-        const esg_status pst = bf2_plan(hl.data(), hr.data(), nq, n, d, sms, true, P);
+        const esg_status pst = bf2_plan(hl.data(), hr.data(), nq, n, d, sms, true, K1, P);
         if (pst != ESG_OK) return pst;
     }
     const std::vector<int32_t> &order = P.order, &item_begin = P.item_begin, &cta_first = P.cta_first;
@@ -1754,14 +1787,15 @@ static esg_status bf2_queries(const PreparedX &X, const float *base, int64_t n, 
             ce = split_norm(queries, nv, d, nk, d_order, nqt * TM, qs, qnorm, qrow, nullptr, stream);
     }
     // lists in 32 or 64 registers-times-lanes
-    const bool l2 = metric == ESG_L2SQ, one = K1 <= 32;
+    const bool l2 = metric == ESG_L2SQ, one = K1 <= 32, two = K1 <= 64;
     auto pick = [&](auto s) -> void (*)(Tc2Args) {
         constexpr bool ST = decltype(s)::value;
         switch (bf2_reg_list(K1)) {
             case 24: return l2 ? tc_knn2_kernel<true, 24, 1, ST> : tc_knn2_kernel<false, 24, 1, ST>;
             case 32: return l2 ? tc_knn2_kernel<true, 32, 1, ST> : tc_knn2_kernel<false, 32, 1, ST>;
         }
-        return l2 ? tc_knn2_kernel<true, 0, 2, ST> : tc_knn2_kernel<false, 0, 2, ST>;
+        return l2 ? (two ? tc_knn2_kernel<true, 0, 2, ST> : tc_knn2_kernel<true, 0, 4, ST>)
+                  : (two ? tc_knn2_kernel<false, 0, 2, ST> : tc_knn2_kernel<false, 0, 4, ST>);
     };
     void (*fn)(Tc2Args) = stream_a ? pick(std::true_type{}) : pick(std::false_type{});
     if (ce == cudaSuccess) ce = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -1790,15 +1824,17 @@ static esg_status bf2_queries(const PreparedX &X, const float *base, int64_t n, 
         esg_prof_end(pidx, stream);
         if (ce == cudaSuccess) {
             const FinishArgs f{base, queries, d, metric, k, K1, part, part_n, d_ib, d_order, d_doff, l, r, dense, qnorm, qrow,
-                               X.xmax,
+                               X.xmax, bf2_serial(d, k) ? 1 : 0,
                                out_ids, out_dist, out_count, redo};
             // many lists per query: two per item, items shared out over the query tiles
             if (n_items > 16 * nqt) {
                 if (one) finish_kernel<1, 16><<<(unsigned)nv, 512, 0, stream>>>(f);
-                else finish_kernel<2, 16><<<(unsigned)nv, 512, 0, stream>>>(f);
+                else if (two) finish_kernel<2, 16><<<(unsigned)nv, 512, 0, stream>>>(f);
+                else finish_kernel<4, 8><<<(unsigned)nv, 256, 0, stream>>>(f);
             } else {
                 if (one) finish_kernel<1, 4><<<(unsigned)nv, 128, 0, stream>>>(f);
-                else finish_kernel<2, 4><<<(unsigned)nv, 128, 0, stream>>>(f);
+                else if (two) finish_kernel<2, 4><<<(unsigned)nv, 128, 0, stream>>>(f);
+                else finish_kernel<4, 4><<<(unsigned)nv, 128, 0, stream>>>(f);
             }
             ce = cudaGetLastError();
         }
@@ -1824,20 +1860,18 @@ static esg_status bf2_queries(const PreparedX &X, const float *base, int64_t n, 
 }
 
 // Pipelined tensor-core path; ESG_ERR_UNSUPPORTED when the shape does not fit
-// (k > 56, or shared memory for fewer than two stages). Each list keeps
-// K1 = k + 12 approximate candidates (k + 8 where the longer list does not
-// fit in shared memory): the certificate needs the exact k-th
+// (k > 120, or shared memory for fewer than two stages). Each list keeps
+// about k + 12 approximate candidates: the certificate needs the exact k-th
 // distance below the approximate K1-th minus the error bound, which holds for
 // nearly every query, and a short list makes the epilogue's filter sharp; the
-// few queries left uncertified run again with 64 candidates.
+// few queries left uncertified run again with a longer list.
 static esg_status bruteforce_tc_v2(const float *base, int64_t n, int32_t d, int metric, const float *queries,
                                    int64_t nq, const int64_t *l, const int64_t *r, int32_t k, int64_t *out_ids,
                                    float *out_dist, int32_t *out_count, cudaStream_t stream) {
-    // k + 12 candidates, at least k + 8 (the longest list the kernel holds
-    // caps it): at 1M x 128, 10k queries, k = 10, lists of k + 8 left 2 queries
-    // uncertified and their second pass cost 0.75 ms of a 5.90 ms call; k + 12
-    // certified all
-    if (k < 1 || k + 8 > ((d + TK - 1) / TK == 1 ? kMaxK1v2 : kMaxK1v2 - 6) || n >= ((int64_t)1 << 31) || d < 1) return ESG_ERR_UNSUPPORTED;
+    // k + 12 candidates (the register lists' 24 or 32 for k up to 20), at least
+    // k + 8 (the longest list the kernel holds caps it): at 1M x 128, 10k
+    // queries, k = 10, lists of k + 8 left 2 queries uncertified, k + 12 certified all
+    if (k < 1 || k + 8 > kMaxK1v2 || n >= ((int64_t)1 << 31) || d < 1) return ESG_ERR_UNSUPPORTED;
     const int K1 = k <= 12 ? 24 : (k <= 20 ? 32 : std::min(k + 12, kMaxK1v2));
     int dev = 0, max_smem = 0, S = 0, n_acc = 0;
     bool stream_a = false, list_smem = false;
@@ -1873,7 +1907,7 @@ static esg_status bruteforce_tc_v2(const float *base, int64_t n, int32_t d, int 
     if (ce != cudaSuccess) { esg_set_error(cudaGetErrorString(ce)); st = ESG_ERR_CUDA; }
     const double t1 = bf_stats() ? bf_host_ms() : 0.0;
     Bf2Plan P;
-    if (st == ESG_OK) st = bf2_plan(hl.data(), hr.data(), nq, n, d, sms, true, P);
+    if (st == ESG_OK) st = bf2_plan(hl.data(), hr.data(), nq, n, d, sms, true, K1, P);
     if (bf_stats()) fprintf(stderr, "tensor-core brute force, host ms: ranges + point prep queued %.3f, plan %.3f\n",
                             t1 - t0, bf_host_ms() - t1);
     if (st == ESG_OK) {
@@ -1903,7 +1937,7 @@ esg_status esg_bruteforce_plan(int64_t n, int32_t d, const int64_t *l, const int
     Bf2Plan P;
     esg_status st = ESG_OK;
     try {
-        st = bf2_plan(l, r, nq, n, d, ctas, false, P);
+        st = bf2_plan(l, r, nq, n, d, ctas, false, 0, P);
     } catch (...) { st = ESG_ERR_OOM; }
     if (st != ESG_OK) {
         if (st == ESG_ERR_UNSUPPORTED) esg_set_error("esg_bruteforce_plan: more than 2^31 covered point tiles");
