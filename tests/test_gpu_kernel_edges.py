@@ -3,6 +3,7 @@ chunks, remainders, the smallest and largest of each range."""
 import numpy as np
 import pytest
 
+import oracle as O
 from oracle import mlp as OM
 
 torch = pytest.importorskip("torch")
@@ -87,3 +88,67 @@ def test_exact_lists_and_dense_rows(d, metric, k):
     pick = list(range(len(edge))) + rng.choice(np.arange(len(edge), nq), 12, replace=False).tolist()
     _check_exact(X.cpu().numpy(), Q.cpu().numpy()[pick], l[pick], r[pick], k, metric, ids.cpu().numpy()[pick],
                  dist.cpu().numpy()[pick], count.cpu().numpy()[pick])
+
+
+@pytest.mark.parametrize("d", [32, 64, 128, 192, 260])
+@pytest.mark.parametrize("metric", ["l2", "ip"])
+@pytest.mark.parametrize("k", [51, 56, 57, 100, 116, 120, 121])
+def test_exact_long_lists(d, metric, k):
+    """Lists of up to 128 (k up to 120, summed in dimension order where the
+    SIMT kernel used to answer) and the SIMT kernel above, over ranges that are
+    dense rows and lists, shorter than k, one point, and at tile edges."""
+    n, nq = 9_001, 140
+    g = torch.Generator(device=DEV).manual_seed(d * 1000 + k)
+    X = torch.randn(n, d, generator=g, device=DEV)
+    Q = torch.randn(nq, d, generator=g, device=DEV)
+    rng = np.random.default_rng(d + k)
+    w = np.exp(rng.uniform(0, np.log(n), nq)).astype(np.int64)
+    l = (rng.random(nq) * (n - w + 1)).astype(np.int64)
+    r = l + w - 1
+    edge = [(0, n - 1), (0, 0), (n - 1, n - 1), (127, 128), (128, 128 + k - 1), (100, 100 + k), (0, 255)]
+    l[:len(edge)], r[:len(edge)] = zip(*edge)
+    ids, dist, count = E.esg_bruteforce_filtered_knn(X, Q, _t(l), _t(r), k, metric)
+    torch.cuda.synchronize()
+    pick = list(range(len(edge))) + rng.choice(np.arange(len(edge), nq), 20, replace=False).tolist()
+    _check_exact(X.cpu().numpy(), Q.cpu().numpy()[pick], l[pick], r[pick], k, metric, ids.cpu().numpy()[pick],
+                 dist.cpu().numpy()[pick], count.cpu().numpy()[pick])
+
+
+@pytest.mark.parametrize("k,d", [(100, 96), (57, 64), (51, 128)])
+def test_exact_long_lists_equal_simt(k, d, monkeypatch):
+    """Where the SIMT kernel used to answer, the lists' answers are its, bit
+    for bit: ids, distances, counts (ranges of list and dense rows)."""
+    n, nq = 300_000, 40
+    g = torch.Generator(device=DEV).manual_seed(k)
+    cen = torch.randn(200, d, generator=g, device=DEV)
+    X = cen[torch.randint(0, 200, (n,), generator=g, device=DEV)] + 0.3 * torch.randn(n, d, generator=g, device=DEV)
+    Q = X[torch.randint(0, n, (nq,), generator=g, device=DEV)] + 0.1 * torch.randn(nq, d, generator=g, device=DEV)
+    rng = np.random.default_rng(k)
+    w = np.exp(rng.uniform(np.log(50), np.log(n), nq)).astype(np.int64)
+    w[:2] = n, n - 1
+    l = (rng.random(nq) * (n - w + 1)).astype(np.int64)
+    a = E.esg_bruteforce_filtered_knn(X, Q, _t(l), _t(l + w - 1), k)
+    monkeypatch.setenv("ESG_BF_SIMT", "1")
+    b = E.esg_bruteforce_filtered_knn(X, Q, _t(l), _t(l + w - 1), k)
+    torch.cuda.synchronize()
+    assert all(torch.equal(x, y) for x, y in zip(a, b))
+
+
+@pytest.mark.parametrize("d,M,efc,n", [(8, 1, 3, 200), (32, 4, 40, 400), (128, 16, 200, 500), (768, 8, 300, 400)])
+@pytest.mark.parametrize("metric", ["l2", "ip"])
+def test_build_one_at_a_time_is_the_oracles(d, M, efc, n, metric):
+    """With rounds of one point the build is the oracle's: the same rows (as
+    sets) on small integer coordinates, whose distances are exact in float32
+    (pools of one and several steps, of rows staged in shared memory wholly
+    and in part; full rows re-selected)."""
+    rng = np.random.default_rng(d + M)
+    X = rng.integers(-20, 21, (n, d)).astype(np.float32)
+    ix = E.esg_build(X, None, M=M, leaf_size=64, n_entries=8, ef_construction=efc, batch_div=1 << 20, metric=metric)
+    adj, _, _ = E.esg_index_export(ix)
+    want = O.build_index(X, np.arange(n, dtype=np.float64), metric, 64, M, efc=efc, n_entries=8).adj
+    assert adj.shape == want.shape
+    for lev in range(ix.L):
+        for p in range(n):
+            got = adj[lev, p]
+            assert np.all(np.diff((got == 0xFFFFFFFF).astype(int)) >= 0)
+            assert set(got.tolist()) == set(np.asarray(want[lev, p], dtype=np.uint32).tolist()), (lev, p)
