@@ -1152,7 +1152,10 @@ __global__ void __launch_bounds__(32 * WQ) finish_kernel(FinishArgs f) {
     for (int h = 0; h < NL; ++h)
         if (h == (max(c, 1) - 1) >> 5) last = R[h];
     last = __shfl_sync(0xffffffffu, last, (max(c, 1) - 1) & 31);
-    bool certified = c > 0;
+    // a list shorter than its range has dropped points at +inf or NaN: theirs are
+    // the exact distances too, unless a norm overflows or an element has no BF16
+    // part (then its row's norm overflows): those queries go to the SIMT kernel
+    bool certified = c > 0 && (m > f.r[q] - f.l[q] || (f.qrownorm[q] < INFINITY && f.xmax[0] < INFINITY));
     if (m == f.K1) {   // the list is full: points may have been left out
         // |approximate - exact| for any point of the range (unit roundoff of
         // BF16 2^-8, of FP32 2^-24): the split residuals and the dropped
@@ -1289,7 +1292,7 @@ struct Bf2Plan;
 static esg_status bf2_queries(const PreparedX &X, const float *base, int64_t n, int32_t d, int metric,
                               const float *queries, int64_t nq, const int64_t *l, const int64_t *r, int32_t k,
                               int K1, int64_t *out_ids, float *out_dist, int32_t *out_count, cudaStream_t stream,
-                              Bf2Plan *given = nullptr);
+                              Bf2Plan *given = nullptr, bool dense_rows = true);
 
 // Queries whose list of K1 candidates could not be certified run again with
 // the longest list that fits the kernel (their own plan, a few query tiles), and
@@ -1528,10 +1531,10 @@ static void bf2_dense(const int64_t *hl, const int64_t *hr, int64_t widest, int6
     std::fill(P.doff.begin(), P.doff.end(), (int64_t)-1);
 }
 
-// `run`: the plan is for the kernel with lists of K1 (dense rows, its restart
-// cost), not for inspection.
+// `run`: the plan is for the kernel with lists of K1 (dense rows where `dense_rows`,
+// its restart cost), not for inspection.
 static esg_status bf2_plan(const int64_t *hl, const int64_t *hr, int64_t nq, int64_t n, int32_t d, int64_t sms,
-                           bool run, int K1, Bf2Plan &P) {
+                           bool run, int K1, Bf2Plan &P, bool dense_rows = true) {
     // sorted by (floor(log2 width), l, query index): a stable LSD radix sort
     // of the valid queries in index order, by 11 bits of l at a time and then
     // by the width class
@@ -1611,7 +1614,7 @@ static esg_status bf2_plan(const int64_t *hl, const int64_t *hr, int64_t nq, int
     {
         std::vector<int32_t> lt(nv), rt(nv), dense(nv, 0);
         const int64_t x = K1 > 32 ? 2 : 1;
-        if (run) bf2_dense(hl, hr, nk <= 2 ? x * kDenseWidth : 0, x * kDenseFloats, P);
+        if (run) bf2_dense(hl, hr, dense_rows && nk <= 2 ? x * kDenseWidth : 0, x * kDenseFloats, P);
         for (int64_t s = 0; s < nv; ++s) {
             lt[s] = (int32_t)(hl[order[s]] / TN);
             rt[s] = (int32_t)(hr[order[s]] / TN);
@@ -1687,11 +1690,12 @@ __global__ void expand_tiles_kernel(const WorkItem *items, const int32_t *span_a
     }
 }
 
-// `given`: a plan already made for these ranges (it is consumed), or null.
+// `given`: a plan already made for these ranges (it is consumed), or null. Where
+// memory is too short for the dense rows' buffer the pass goes without it.
 static esg_status bf2_queries(const PreparedX &X, const float *base, int64_t n, int32_t d, int metric,
                               const float *queries, int64_t nq, const int64_t *l, const int64_t *r, int32_t k,
                               int K1, int64_t *out_ids, float *out_dist, int32_t *out_count, cudaStream_t stream,
-                              Bf2Plan *given) {
+                              Bf2Plan *given, bool dense_rows) {
     if (nq == 0) return ESG_OK;
     const double h0 = bf_stats() ? bf_host_ms() : 0.0;
     const int nk = (d + TK - 1) / TK;
@@ -1712,7 +1716,7 @@ static esg_status bf2_queries(const PreparedX &X, const float *base, int64_t n, 
         ESG_CUDA_TRY(cudaMemcpyAsync(hl.data(), l, sizeof(int64_t) * nq, cudaMemcpyDeviceToHost, stream));
         ESG_CUDA_TRY(cudaMemcpyAsync(hr.data(), r, sizeof(int64_t) * nq, cudaMemcpyDeviceToHost, stream));
         ESG_CUDA_TRY(cudaStreamSynchronize(stream));
-        const esg_status pst = bf2_plan(hl.data(), hr.data(), nq, n, d, sms, true, K1, P);
+        const esg_status pst = bf2_plan(hl.data(), hr.data(), nq, n, d, sms, true, K1, P, dense_rows);
         if (pst != ESG_OK) return pst;
     }
     const std::vector<int32_t> &order = P.order, &item_begin = P.item_begin, &cta_first = P.cta_first;
@@ -1732,7 +1736,13 @@ static esg_status bf2_queries(const PreparedX &X, const float *base, int64_t n, 
                    al(sizeof(int64_t) * std::max<int64_t>(nv, 1)) + al(sizeof(float) * P.dense) +
                    al(sizeof(int32_t) * n_spans) + al(sizeof(int64_t) * n_spans) + al(sizeof(int32_t) * (nqt + 1));
     unsigned char *scratch = nullptr;
-    ESG_CUDA_TRY(esg_malloc_async((void **)&scratch, bytes, stream));
+    const cudaError_t me = esg_malloc_async((void **)&scratch, bytes, stream);
+    if (me == cudaErrorMemoryAllocation && P.dense > 0) {
+        cudaGetLastError();
+        return bf2_queries(X, base, n, d, metric, queries, nq, l, r, k, K1, out_ids, out_dist, out_count, stream,
+                           nullptr, false);
+    }
+    ESG_CUDA_TRY(me);
     unsigned char *p = scratch;
     auto take = [&](size_t b) { unsigned char *q = p; p += al(b); return q; };
     unsigned char *qs = take((size_t)std::max<int64_t>(nqt, 1) * nk * STAGE);
@@ -1907,7 +1917,14 @@ static esg_status bruteforce_tc_v2(const float *base, int64_t n, int32_t d, int 
     if (ce != cudaSuccess) { esg_set_error(cudaGetErrorString(ce)); st = ESG_ERR_CUDA; }
     const double t1 = bf_stats() ? bf_host_ms() : 0.0;
     Bf2Plan P;
-    if (st == ESG_OK) st = bf2_plan(hl.data(), hr.data(), nq, n, d, sms, true, K1, P);
+    if (st == ESG_OK) {
+        try {
+            st = bf2_plan(hl.data(), hr.data(), nq, n, d, sms, true, K1, P);
+        } catch (...) {
+            esg_set_error("tensor-core brute force: out of memory (host plan)");
+            st = ESG_ERR_OOM;
+        }
+    }
     if (bf_stats()) fprintf(stderr, "tensor-core brute force, host ms: ranges + point prep queued %.3f, plan %.3f\n",
                             t1 - t0, bf_host_ms() - t1);
     if (st == ESG_OK) {
@@ -1919,11 +1936,31 @@ static esg_status bruteforce_tc_v2(const float *base, int64_t n, int32_t d, int 
 }
 
 // Tensor-core path of esg_bruteforce_filtered_knn; returns ESG_ERR_UNSUPPORTED
-// when the shape is outside both versions (the caller then uses the SIMT kernel).
+// when the shape is outside it (the caller then uses the SIMT kernel). Where the
+// SIMT kernel gives the same answers bit for bit (bf2_serial), it also serves
+// calls that this path cannot: it needs no scratch memory and no host
+// synchronisation, so it runs when memory is short and under stream capture.
 esg_status esg_bruteforce_tc(const float *base, int64_t n, int32_t d, int metric, const float *queries,
                              int64_t nq, const int64_t *l, const int64_t *r, int32_t k, int64_t *out_ids,
                              float *out_dist, int32_t *out_count, cudaStream_t stream) {
-    return bruteforce_tc_v2(base, n, d, metric, queries, nq, l, r, k, out_ids, out_dist, out_count, stream);
+    const bool simt_too = bf2_serial(d, k);
+    if (simt_too) {
+        cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(stream, &cs) != cudaSuccess) cudaGetLastError();
+        if (cs != cudaStreamCaptureStatusNone) return ESG_ERR_UNSUPPORTED;
+    }
+    esg_status st;
+    try {
+        st = bruteforce_tc_v2(base, n, d, metric, queries, nq, l, r, k, out_ids, out_dist, out_count, stream);
+    } catch (...) {
+        esg_set_error("tensor-core brute force: out of memory (host)");
+        st = ESG_ERR_OOM;
+    }
+    if (simt_too && st == ESG_ERR_OOM) {
+        cudaGetLastError();   // the failed allocation's
+        st = ESG_ERR_UNSUPPORTED;
+    }
+    return st;
 }
 
 esg_status esg_bruteforce_plan(int64_t n, int32_t d, const int64_t *l, const int64_t *r, int64_t nq,

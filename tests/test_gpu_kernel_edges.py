@@ -152,3 +152,54 @@ def test_build_one_at_a_time_is_the_oracles(d, M, efc, n, metric):
             got = adj[lev, p]
             assert np.all(np.diff((got == 0xFFFFFFFF).astype(int)) >= 0)
             assert set(got.tolist()) == set(np.asarray(want[lev, p], dtype=np.uint32).tolist()), (lev, p)
+
+
+def _long_list_case(nq=70, n=20_000, d=64, k=100):
+    g = torch.Generator(device=DEV).manual_seed(5)
+    X = torch.randn(n, d, generator=g, device=DEV)
+    Q = torch.randn(nq, d, generator=g, device=DEV)
+    rng = np.random.default_rng(5)
+    w = np.exp(rng.uniform(0, np.log(n), nq)).astype(np.int64)
+    l = (rng.random(nq) * (n - w + 1)).astype(np.int64)
+    return X, Q, _t(l), _t(l + w - 1), k
+
+
+@pytest.mark.parametrize("k", [10, 60])
+def test_exact_short_range_keeps_points_without_bf16_parts(k, monkeypatch):
+    """A finite element above the largest BF16 leaves its row without an
+    approximate distance; a range shorter than the list still holds the row."""
+    X, Q, _, _, _ = _long_list_case(nq=4, n=300)
+    X[7, 0] = 3.4e38
+    Q[:, 0] = 1e-30
+    l, r = _t(np.array([0, 7, 3, 100])), _t(np.array([7, 7, 20, 111]))
+    a = E.esg_bruteforce_filtered_knn(X, Q, l, r, k, "ip")
+    monkeypatch.setenv("ESG_BF_SIMT", "1")
+    b = E.esg_bruteforce_filtered_knn(X, Q, l, r, k, "ip")
+    assert a[2].tolist()[:2] == [8, 1] and torch.equal(a[2], b[2]) and torch.equal(a[0], b[0])
+
+
+def test_exact_long_lists_under_capture():
+    """A call the SIMT kernel can answer too is captured like any launch."""
+    X, Q, l, r, k = _long_list_case()
+    want = E.esg_bruteforce_filtered_knn(X, Q, l, r, k)
+    out = tuple(torch.empty_like(t) for t in want)
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        E.esg_bruteforce_filtered_knn(X, Q, l, r, k, out=out)
+    for t in out:
+        t.zero_()
+    g.replay()
+    torch.cuda.synchronize()
+    assert all(torch.equal(x, y) for x, y in zip(want, out))
+
+
+@pytest.mark.parametrize("k,kth", [(100, 1), (100, 2), (10, 2)])
+def test_exact_without_memory_for_scratch(k, kth, monkeypatch):
+    """Short of memory for the point blocks, lists of k = 100 come from the SIMT
+    kernel; short of it for the dense rows, every range keeps lists."""
+    X, Q, l, r, _ = _long_list_case()
+    want = E.esg_bruteforce_filtered_knn(X, Q, l, r, k)
+    monkeypatch.setenv("ESG_FAULT_ALLOC", str(kth))
+    got = E.esg_bruteforce_filtered_knn(X, Q, l, r, k)
+    torch.cuda.synchronize()
+    assert all(torch.equal(x, y) for x, y in zip(want, got))
