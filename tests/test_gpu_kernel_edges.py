@@ -203,3 +203,32 @@ def test_exact_without_memory_for_scratch(k, kth, monkeypatch):
     got = E.esg_bruteforce_filtered_knn(X, Q, l, r, k)
     torch.cuda.synchronize()
     assert all(torch.equal(x, y) for x, y in zip(want, got))
+
+
+@pytest.mark.parametrize("M", [8, 16, 32])
+@pytest.mark.parametrize("width", [1, 2])
+@pytest.mark.parametrize("rows", ["f32", "bf16"])
+def test_search_merges_every_batch_size(M, width, rows):
+    """Rows of 16, 32 and 64 neighbours, one or two expanded at a time: admitted
+    batches from one candidate to 128, merged 32 at a time. With a beam that holds
+    the whole set, answers are the exact ones (of the reachable points: recall
+    0.99), each once, ascending, at its float64 distance."""
+    n, nq, k = 700, 40, 100
+    rng = np.random.default_rng(M)
+    X = rng.standard_normal((n, 32)).astype(np.float32)
+    ix = E.esg_build(X, None, M=M, leaf_size=64, n_entries=16, storage=rows)
+    q = rng.standard_normal((nq, 32)).astype(np.float32)
+    w = np.exp(rng.uniform(np.log(k), np.log(n), nq)).astype(np.int64)
+    l = (rng.random(nq) * (n - w + 1)).astype(np.int64)
+    ids, dist, count, status = (t.cpu().numpy() for t in E.esg_search_batch(
+        ix, _t(q), _t(l), _t(l + w - 1), None, k,
+        params=E.search_params(704, traversal=rows, width=width))[:4])
+    hit = 0
+    for i in range(nq):
+        got = ids[i, :count[i]]
+        assert len(set(got.tolist())) == len(got) and got.min() >= l[i] and got.max() < l[i] + w[i]
+        d = ((X.astype(np.float64) - q[i]) ** 2).sum(1)
+        assert np.allclose(dist[i, :count[i]], d[got], rtol=1e-5) and np.all(np.diff(dist[i, :count[i]]) >= 0)
+        want = np.argsort(d[l[i]:l[i] + w[i]], kind="stable")[:k] + l[i]
+        hit += len(set(want.tolist()) & set(got.tolist()))
+    assert hit >= 0.99 * nq * k
