@@ -128,6 +128,9 @@ __device__ __forceinline__ Key make_key(float d, uint32_t row) {
     const uint32_t b = __float_as_uint(d);
     return ((Key)(b ^ ((uint32_t)((int32_t)b >> 31) | 0x80000000u)) << 32) | row;
 }
+// An exact distance's key: both zeros are one distance, ordered by the row
+// alone (an inner product that underflows from below is -0, others +0).
+__device__ __forceinline__ Key exact_key(float d, uint32_t row) { return make_key(d == 0.f ? 0.f : d, row); }
 __device__ __forceinline__ float key_dist(Key k) {
     const uint32_t b = (uint32_t)(k >> 32);
     return __uint_as_float((b & 0x80000000u) ? (b ^ 0x80000000u) : ~b);
@@ -1104,7 +1107,7 @@ __global__ void __launch_bounds__(32 * WQ) finish_kernel(FinishArgs f) {
                     acc = fmaf(qv.z, x.z, acc); acc = fmaf(qv.w, x.w, acc);
                 }
             }
-            s_keys[1][e] = make_key(f.metric == ESG_L2SQ ? acc : -acc, id);
+            s_keys[1][e] = exact_key(f.metric == ESG_L2SQ ? acc : -acc, id);
         }
     } else
     // exact distances: lane j of a warp sums the dimensions j, j + 32, ...,
@@ -1137,7 +1140,7 @@ __global__ void __launch_bounds__(32 * WQ) finish_kernel(FinishArgs f) {
         for (int c = 0; c < 4; ++c) {
             acc[c] = warp_sum_group(acc[c], 32);
             if (lane == 0 && e0 + c < m)
-                s_keys[1][e0 + c] = make_key(f.metric == ESG_L2SQ ? acc[c] : -acc[c], id[c]);
+                s_keys[1][e0 + c] = exact_key(f.metric == ESG_L2SQ ? acc[c] : -acc[c], id[c]);
         }
     }
     __syncthreads();
@@ -1173,12 +1176,14 @@ __global__ void __launch_bounds__(32 * WQ) finish_kernel(FinishArgs f) {
         const double dk = (double)key_dist(last);
         certified = dk + fabs(dk) * f.d * 0x1p-23 < bound;
     }
+    const float zero = f.metric == ESG_L2SQ ? 0.f : -0.f;   // a negated product of 0 is -0
 #pragma unroll
     for (int h = 0; h < NL; ++h) {
         const int e = lane + 32 * h;
         if (e < f.k) {
             f.out_ids[q * f.k + e] = e < c ? (int64_t)(uint32_t)R[h] : -1;
-            f.out_dist[q * f.k + e] = e < c ? key_dist(R[h]) : INFINITY;
+            const float x = key_dist(R[h]);
+            f.out_dist[q * f.k + e] = e < c ? (x == 0.f ? zero : x) : INFINITY;
         }
     }
     if (lane == 0) { f.out_count[q] = c; f.redo[q] = certified ? 0 : 1; }

@@ -232,3 +232,19 @@ def test_search_merges_every_batch_size(M, width, rows):
         want = np.argsort(d[l[i]:l[i] + w[i]], kind="stable")[:k] + l[i]
         hit += len(set(want.tolist()) & set(got.tolist()))
     assert hit >= 0.99 * nq * k
+
+
+@pytest.mark.parametrize("k", [10, 60])
+def test_exact_equal_zeros_order_by_row(k):
+    """Inner products that underflow from either side are 0, a tie of all rows:
+    the answer is the first rows, in order."""
+    X, Q, _, _, _ = _long_list_case(nq=3, d=32)
+    X[:] = 1e-30
+    X[::3] = -1e-30
+    Q[:] = 1e-30
+    l = np.array([0, 5, 0])
+    r = np.array([19, 24, len(X) - 1])
+    ids, dist, count = E.esg_bruteforce_filtered_knn(X, Q, _t(l), _t(r), k, "ip")
+    for i, c in enumerate((min(k, 20), min(k, 20), k)):
+        assert count[i] == c and torch.all(dist[i, :c] == 0)
+        assert ids[i, :c].tolist() == list(range(l[i], l[i] + c))
