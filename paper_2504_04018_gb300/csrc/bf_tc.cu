@@ -1176,6 +1176,10 @@ __global__ void __launch_bounds__(32 * WQ) finish_kernel(FinishArgs f) {
         const double dk = (double)key_dist(last);
         certified = dk + fabs(dk) * f.d * 0x1p-23 < bound;
     }
+    // the largest product of norms whose BF16 parts' products cannot overflow
+    // (each part is up to 2^-8 above its element): beyond it an inner product
+    // that FP32 holds may have been dropped as infinite
+    if (f.metric == ESG_IP && !((double)f.qrownorm[q] * f.xmax[0] < 0x1.fcp127)) certified = false;
     const float zero = f.metric == ESG_L2SQ ? 0.f : -0.f;   // a negated product of 0 is -0
 #pragma unroll
     for (int h = 0; h < NL; ++h) {

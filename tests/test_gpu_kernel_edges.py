@@ -248,3 +248,18 @@ def test_exact_equal_zeros_order_by_row(k):
     for i, c in enumerate((min(k, 20), min(k, 20), k)):
         assert count[i] == c and torch.all(dist[i, :c] == 0)
         assert ids[i, :c].tolist() == list(range(l[i], l[i] + c))
+
+
+@pytest.mark.parametrize("k", [10, 60])
+def test_exact_inner_products_near_the_largest_float(k, monkeypatch):
+    """A product that FP32 holds, of elements whose BF16 parts' product does not."""
+    X, Q, _, _, _ = _long_list_case(nq=3)
+    X[3] = 0
+    Q[0] = 0
+    X[3, 0], Q[0, 0] = -1.843e19, 1.843e19
+    l, r = _t(np.array([0, 0, 0])), _t(np.array([9, 299, len(X) - 1]))
+    a = E.esg_bruteforce_filtered_knn(X, Q, l, r, k, "ip")
+    assert a[2].tolist() == [10, k, k] and 3 in a[0][0].tolist()
+    monkeypatch.setenv("ESG_BF_SIMT", "1")
+    b = E.esg_bruteforce_filtered_knn(X, Q, l, r, k, "ip")
+    assert torch.equal(a[2], b[2]) and torch.equal(a[0], b[0])
