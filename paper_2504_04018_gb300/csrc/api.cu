@@ -8,6 +8,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <mutex>
+#include <new>
 #include <numeric>
 #include <string>
 #include <vector>
@@ -102,17 +103,34 @@ cudaMemPool_t esg_scratch_pool() {
     return pools[dev];
 }
 
+// Whether this is the K-th call since the environment variable `name` was set to K.
+namespace {
+struct FaultCounter {
+    const char *name;
+    std::mutex mu;
+    std::string seen;
+    long long count = 0;
+    explicit FaultCounter(const char *n) : name(n) {}
+    bool hit() {
+        const char *v = getenv(name);
+        const std::string cur = v ? v : "";
+        std::lock_guard<std::mutex> lk(mu);
+        if (cur != seen) { seen = cur; count = 0; }   // a new value starts a new count
+        if (cur.empty()) return false;
+        const long long k = atoll(cur.c_str());
+        return k >= 1 && ++count == k;
+    }
+};
+}  // namespace
+
 bool esg_fault_alloc() {
-    static std::mutex mu;
-    static std::string seen;
-    static long long count = 0;
-    const char *v = getenv("ESG_FAULT_ALLOC");
-    const std::string cur = v ? v : "";
-    std::lock_guard<std::mutex> lk(mu);
-    if (cur != seen) { seen = cur; count = 0; }   // a new value starts a new count
-    if (cur.empty()) return false;
-    const long long k = atoll(cur.c_str());
-    return k >= 1 && ++count == k;
+    static FaultCounter c("ESG_FAULT_ALLOC");
+    return c.hit();
+}
+
+void esg_fault_host() {
+    static FaultCounter c("ESG_FAULT_HOST_ALLOC");
+    if (c.hit()) throw std::bad_alloc();
 }
 
 esg_status esg_check_search_params(const esg_search_params &p, const char *who) {

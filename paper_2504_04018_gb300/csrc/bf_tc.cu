@@ -1205,9 +1205,26 @@ __global__ void invalid_kernel(const int64_t *l, const int64_t *r, int64_t nq, i
 
 }  // namespace
 
+// Device scratch of a call, given back on its stream whichever way the call
+// ends (a host allocation may throw with scratch held and work queued).
+struct Scratch {
+    unsigned char *p = nullptr;
+    cudaStream_t stream;
+    explicit Scratch(cudaStream_t s) : stream(s) {}
+    Scratch(const Scratch &) = delete;
+    Scratch &operator=(const Scratch &) = delete;
+    ~Scratch() { release(); }
+    cudaError_t alloc(size_t bytes) { return esg_malloc_async((void **)&p, bytes, stream); }
+    void release() {
+        if (p) cudaFreeAsync(p, stream);
+        p = nullptr;
+    }
+};
+
 // Waits for the pass and returns the queries it left uncertified.
 static esg_status read_uncertified(int64_t nq, int K1, const int32_t *redo, const int32_t *err, cudaStream_t stream,
                                    std::vector<int64_t> &idx) {
+    esg_fault_host();
     std::vector<int32_t> h_redo(nq);
     int32_t h_err = 0;
     cudaError_t ce = cudaMemcpyAsync(h_redo.data(), redo, sizeof(int32_t) * nq, cudaMemcpyDeviceToHost, stream);
@@ -1317,9 +1334,9 @@ static esg_status bf2_escalate(const PreparedX &X, const float *base, int64_t n,
     auto al = [](size_t x) { return (x + 255) & ~(size_t)255; };
     const size_t bytes = al(sizeof(int64_t) * m) + al(sizeof(float) * m * d) + 2 * al(sizeof(int64_t) * m) +
                          al(sizeof(int64_t) * m * k) + al(sizeof(float) * m * k) + al(sizeof(int32_t) * m);
-    unsigned char *sc = nullptr;
-    ESG_CUDA_TRY(esg_malloc_async((void **)&sc, bytes, stream));
-    unsigned char *p = sc;
+    Scratch sc(stream);
+    ESG_CUDA_TRY(sc.alloc(bytes));
+    unsigned char *p = sc.p;
     int64_t *didx = (int64_t *)p; p += al(sizeof(int64_t) * m);
     float *Qg = (float *)p; p += al(sizeof(float) * m * d);
     int64_t *lg = (int64_t *)p; p += al(sizeof(int64_t) * m);
@@ -1343,7 +1360,6 @@ static esg_status bf2_escalate(const PreparedX &X, const float *base, int64_t n,
     // the host index vector must outlive the copy above
     const cudaError_t se = cudaStreamSynchronize(stream);
     if (st == ESG_OK && se != cudaSuccess) { esg_set_error(cudaGetErrorString(se)); st = ESG_ERR_CUDA; }
-    cudaFreeAsync(sc, stream);
     return st;
 }
 
@@ -1744,15 +1760,15 @@ static esg_status bf2_queries(const PreparedX &X, const float *base, int64_t n, 
                    al(sizeof(int32_t) * 2 * ni1 * TM) + al(sizeof(int32_t) * nq) + al(sizeof(int32_t) * 4) +
                    al(sizeof(int64_t) * std::max<int64_t>(nv, 1)) + al(sizeof(float) * P.dense) +
                    al(sizeof(int32_t) * n_spans) + al(sizeof(int64_t) * n_spans) + al(sizeof(int32_t) * (nqt + 1));
-    unsigned char *scratch = nullptr;
-    const cudaError_t me = esg_malloc_async((void **)&scratch, bytes, stream);
+    Scratch scratch(stream);
+    const cudaError_t me = scratch.alloc(bytes);
     if (me == cudaErrorMemoryAllocation && P.dense > 0) {
         cudaGetLastError();
         return bf2_queries(X, base, n, d, metric, queries, nq, l, r, k, K1, out_ids, out_dist, out_count, stream,
                            nullptr, false);
     }
     ESG_CUDA_TRY(me);
-    unsigned char *p = scratch;
+    unsigned char *p = scratch.p;
     auto take = [&](size_t b) { unsigned char *q = p; p += al(b); return q; };
     unsigned char *qs = take((size_t)std::max<int64_t>(nqt, 1) * nk * STAGE);
     float *qnorm = (float *)take(sizeof(float) * nq);
@@ -1788,6 +1804,7 @@ static esg_status bf2_queries(const PreparedX &X, const float *base, int64_t n, 
             ce = cudaMemcpyAsync(d_span_first, P.spans.first.data(), sizeof(int32_t) * (nqt + 1),
                                  cudaMemcpyHostToDevice, stream);
         if (ce == cudaSuccess) {
+            esg_fault_host();
             std::vector<int32_t> c(n_items);
             for (int64_t i = 0; i < n_items; ++i) c[i] = items[i].cnt;
             std::nth_element(c.begin(), c.begin() + n_items * 3 / 4, c.end());
@@ -1868,7 +1885,7 @@ static esg_status bf2_queries(const PreparedX &X, const float *base, int64_t n, 
     const double h1 = bf_stats() ? bf_host_ms() : 0.0;
     if (st == ESG_OK)
         st = read_uncertified(nq, K1, redo, err, stream, left);
-    cudaFreeAsync(scratch, stream);
+    scratch.release();
     const double h2 = bf_stats() ? bf_host_ms() : 0.0;
     if (st == ESG_OK && !left.empty())
         st = bf2_escalate(X, base, n, d, metric, queries, nq, l, r, k, K1, left, out_ids, out_dist, out_count, stream);
@@ -1912,9 +1929,9 @@ static esg_status bruteforce_tc_v2(const float *base, int64_t n, int32_t d, int 
     ESG_CUDA_TRY(cudaStreamSynchronize(stream));
     auto al = [](size_t x) { return (x + 255) & ~(size_t)255; };
     const size_t bytes = al((size_t)xt * nk * STAGE) + al(sizeof(float) * xt * TN) + al(sizeof(float) * 4);
-    unsigned char *scratch = nullptr;
-    ESG_CUDA_TRY(esg_malloc_async((void **)&scratch, bytes, stream));
-    unsigned char *p = scratch;
+    Scratch scratch(stream);
+    ESG_CUDA_TRY(scratch.alloc(bytes));
+    unsigned char *p = scratch.p;
     unsigned char *xs = p; p += al((size_t)xt * nk * STAGE);
     float *xnorm = (float *)p; p += al(sizeof(float) * xt * TN);   // past n: never in a range
     float *xmax = (float *)p;
@@ -1940,7 +1957,6 @@ static esg_status bruteforce_tc_v2(const float *base, int64_t n, int32_t d, int 
         const PreparedX X{xs, xnorm, xmax};
         st = bf2_queries(X, base, n, d, metric, queries, nq, l, r, k, K1, out_ids, out_dist, out_count, stream, &P);
     }
-    cudaFreeAsync(scratch, stream);
     return st;
 }
 

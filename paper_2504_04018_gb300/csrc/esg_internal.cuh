@@ -40,6 +40,9 @@ inline cudaError_t esg_malloc(void **p, size_t bytes) {
     if (esg_fault_alloc()) { *p = nullptr; return cudaErrorMemoryAllocation; }
     return cudaMalloc(p, bytes);
 }
+// The same for host memory: with ESG_FAULT_HOST_ALLOC=K, the K-th of the marked
+// host allocations after that value was set throws std::bad_alloc.
+void esg_fault_host();
 // Stream-ordered scratch comes from the library's own memory pool on the
 // current device, which keeps up to ESG_POOL_KEEP_MB (default 8192) MiB of
 // freed memory mapped between calls (the default pool returns it at every

@@ -1,5 +1,9 @@
 """Kernels at the sizes where their tiling can go wrong: edges of tiles and
 chunks, remainders, the smallest and largest of each range."""
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 
@@ -263,3 +267,43 @@ def test_exact_inner_products_near_the_largest_float(k, monkeypatch):
     monkeypatch.setenv("ESG_BF_SIMT", "1")
     b = E.esg_bruteforce_filtered_knn(X, Q, l, r, k, "ip")
     assert torch.equal(a[2], b[2]) and torch.equal(a[0], b[0])
+
+
+_HOST_FAILURE = """
+import os, torch
+import paper_2504_04018_gb300 as E
+g = torch.Generator(device="cuda").manual_seed(1)
+X = torch.randn(200_000, 128, generator=g, device="cuda")
+Q = torch.randn(300, 128, generator=g, device="cuda")
+l = torch.zeros(300, dtype=torch.int64, device="cuda")
+r = l + 199_999
+want = {k: E.esg_bruteforce_filtered_knn(X, Q, l, r, k) for k in (10, 100)}
+def used():
+    torch.cuda.synchronize()
+    free, total = torch.cuda.mem_get_info()
+    return total - free
+before = used()
+for k in (10, 100):
+    for kth in ("1", "2"):
+        os.environ["ESG_FAULT_HOST_ALLOC"] = kth
+        try:
+            got = E.esg_bruteforce_filtered_knn(X, Q, l, r, k)
+            assert k == 100 and all(torch.equal(a, b) for a, b in zip(got, want[k]))
+        except E.EsgError as e:
+            assert k == 10 and "out of memory" in str(e), str(e)
+        del os.environ["ESG_FAULT_HOST_ALLOC"]
+        E.esg_bruteforce_filtered_knn(X, Q, l, r, k)
+after = used()
+assert after <= before + (8 << 20), (before, after)
+print("ok")
+"""
+
+
+def test_exact_host_failure_gives_scratch_back():
+    """A host allocation that fails with device scratch held and work queued: the
+    call fails (or answers through the SIMT kernel) and its scratch, 0.1 GB, is
+    given back. In a process whose pool keeps nothing mapped."""
+    env = dict(os.environ, ESG_POOL_KEEP_MB="0")
+    out = subprocess.run([sys.executable, "-c", _HOST_FAILURE], env=env, capture_output=True, text=True, timeout=300,
+                         cwd=os.path.dirname(os.path.dirname(os.path.abspath(__file__))))
+    assert out.returncode == 0 and out.stdout.strip().endswith("ok"), out.stderr[-2000:]
