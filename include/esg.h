@@ -517,9 +517,9 @@ esg_status esg_bruteforce_filtered_knn(const float *base, int64_t n, int32_t d, 
  * contiguous shares (fewer when there are fewer covered tiles) of about equal
  * estimated cost: tiles + 6.25 (2 / ceil(d / 64))^2 per (query, work item)
  * pair in which the query covers one of the item's tiles; a share is split
- * into work items at query-tile boundaries. A search plans the same order and
- * tiles; its cuts weigh a query whose range begins inside a work item more than
- * one whose list starts with it, and narrow ranges by their tiles.
+ * into work items at query-tile boundaries. This is the plan of plain lists; a
+ * search cuts the same order and tiles by the weights of its own kernel
+ * (esg_bruteforce_search_plan).
  *  n, d       points and dimension of the search (d sets the cost weight);
  *  l, r       host [nq] int64 inclusive ranges;
  *  ctas       CTAs to plan for (the kernel uses one per SM);
@@ -535,6 +535,28 @@ esg_status esg_bruteforce_filtered_knn(const float *base, int64_t n, int32_t d, 
 esg_status esg_bruteforce_plan(int64_t n, int32_t d, const int64_t *l, const int64_t *r, int64_t nq,
                                int32_t ctas, int64_t *sizes, int32_t *order, int32_t *tiles,
                                int32_t *items, int32_t *cta_first);
+
+/*
+ * The plan an esg_bruteforce_filtered_knn call on the tensor-core path makes
+ * (for inspection and tests, no GPU work): order, items and shares as above.
+ * Up to 128 dimensions, queries whose ranges hold at most W points write their
+ * distances to rows of one buffer ("dense rows") instead of keeping lists: W =
+ * 131,072 and a buffer of 2^28 floats, both doubled past k = 20, W halved until
+ * the rows fit. The shares balance tiles + c (16 per query with a list whose
+ * range begins inside the work item, 0.5 per one that begins before it) +
+ * 0.0104 per dense query and tile, all three weights times 2 / ceil(d / 64) (its
+ * third power past 128 dimensions), c = (k + 12) / 24 past k = 20 (k + 12 at
+ * most 128), else 1. A work item's tiles begin at the first one at or after a
+ * multiple of the period and wrap around.
+ *  k          1..120; n, d, l, r, ctas as above;
+ *  sizes      host [6] out: V, T, I, G, floats of the dense rows' buffer, period;
+ *  order, items, cta_first  as above; tiles in the order the CTAs take them;
+ *  dense      host [V] out or NULL: first float of the query's dense row at its
+ *             position (room for points l & ~3 to r | 3), -1 for lists.
+ */
+esg_status esg_bruteforce_search_plan(int64_t n, int32_t d, int32_t k, const int64_t *l, const int64_t *r,
+                                      int64_t nq, int32_t ctas, int64_t *sizes, int32_t *order,
+                                      int32_t *tiles, int32_t *items, int32_t *cta_first, int64_t *dense);
 
 /*
  * Map attribute value ranges [lo, hi] to inclusive rank ranges [l, r] on the

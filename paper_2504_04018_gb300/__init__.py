@@ -19,6 +19,7 @@ from . import _build_lib
 __all__ = [
     "load_library", "Index", "esg_build", "esg_index_import", "esg_index_export", "esg_free",
     "esg_decompose_batch", "esg_search_batch", "esg_bruteforce_filtered_knn", "esg_bruteforce_plan",
+    "esg_bruteforce_search_plan",
     "esg_attr_to_rank_range", "esg_save", "esg_load", "EsgError", "METRIC", "STORAGE",
     "PIECE_GRAPH", "PIECE_SCAN", "Q_INVALID", "Q_TRUNCATED", "Q_OVERFLOW",
 ]
@@ -32,7 +33,8 @@ Q_INVALID, Q_TRUNCATED, Q_OVERFLOW = 1, 2, 4
 EXPORTED = [
     "esg_build_params_default", "esg_search_params_default", "esg_build", "esg_index_import",
     "esg_index_info", "esg_index_layout", "esg_index_export", "esg_free", "esg_decompose_batch", "esg_search_batch",
-    "esg_bruteforce_filtered_knn", "esg_bruteforce_plan", "esg_attr_to_rank_range", "esg_save", "esg_load",
+    "esg_bruteforce_filtered_knn", "esg_bruteforce_plan", "esg_bruteforce_search_plan", "esg_attr_to_rank_range",
+    "esg_save", "esg_load",
     "esg_status_str", "esg_last_error", "esg_profile_enable", "esg_profile_read", "esg_profile_tensor_work",
     "esg_index_export_storage", "esg_index_add_storage", "esg_batch_create", "esg_batch_buffers",
     "esg_batch_run", "esg_batch_free", "esg_autotune", "esg_search_batch_noalloc",
@@ -110,6 +112,7 @@ def load_library(build_if_missing: bool = True) -> ctypes.CDLL:
                                                 _P, _P]
     lib.esg_attr_to_rank_range.argtypes = [_P, _P, _P, _I64, _P, _P]
     lib.esg_bruteforce_plan.argtypes = [_I64, _I32, _P, _P, _I64, _I32, _P, _P, _P, _P, _P]
+    lib.esg_bruteforce_search_plan.argtypes = [_I64, _I32, _I32, _P, _P, _I64, _I32, _P, _P, _P, _P, _P, _P]
     lib.esg_save.argtypes = [_P, ctypes.c_char_p]
     lib.esg_load.argtypes = [ctypes.c_char_p, ctypes.POINTER(_P)]
     lib.esg_profile_enable.argtypes = [_I32]
@@ -469,6 +472,26 @@ def esg_bruteforce_plan(n: int, d: int, l: np.ndarray, r: np.ndarray, ctas: int 
     _check(lib.esg_bruteforce_plan(*args, _np_ptr(sizes), _np_ptr(order), _np_ptr(tiles), _np_ptr(items),
                                    _np_ptr(cta_first)), "esg_bruteforce_plan")
     return order, tiles, items, cta_first
+
+
+def esg_bruteforce_search_plan(n: int, d: int, k: int, l: np.ndarray, r: np.ndarray, ctas: int = 152):
+    """The plan a tensor-core exact search makes (no GPU work): returns (order
+    [V], tiles [T], items [I, 4], cta_first [G + 1]) as int32 arrays, dense [V]
+    int64, the dense rows' floats and the tiles' period."""
+    lib = load_library()
+    l = np.ascontiguousarray(l, dtype=np.int64)
+    r = np.ascontiguousarray(r, dtype=np.int64)
+    sizes = np.zeros(6, dtype=np.int64)
+    args = (n, d, k, _np_ptr(l), _np_ptr(r), l.shape[0], ctas)
+    _check(lib.esg_bruteforce_search_plan(*args, _np_ptr(sizes), None, None, None, None, None),
+           "esg_bruteforce_search_plan")
+    order, tiles = np.empty(sizes[0], dtype=np.int32), np.empty(sizes[1], dtype=np.int32)
+    items = np.empty((sizes[2], 4), dtype=np.int32)
+    cta_first = np.empty(sizes[3] + 1, dtype=np.int32)
+    dense = np.empty(sizes[0], dtype=np.int64)
+    _check(lib.esg_bruteforce_search_plan(*args, _np_ptr(sizes), _np_ptr(order), _np_ptr(tiles), _np_ptr(items),
+                                          _np_ptr(cta_first), _np_ptr(dense)), "esg_bruteforce_search_plan")
+    return order, tiles, items, cta_first, dense, int(sizes[4]), int(sizes[5])
 
 
 def esg_save(index: Index, path: str):

@@ -1246,6 +1246,11 @@ static esg_status read_uncertified(int64_t nq, int K1, const int32_t *redo, cons
 // the lanes: a call's rounding stays what it was.
 static bool bf2_serial(int32_t d, int k) { return k + 8 > ((d + TK - 1) / TK == 1 ? 64 : 58); }
 
+// List length for k: k + 12 candidates (the register lists' 24 or 32 for k up to
+// 20), at least k + 8 (the longest list the kernel holds caps it). At 1M x 128,
+// 10k queries, k = 10, lists of k + 8 left 2 queries uncertified, k + 12 certified all.
+static int bf2_list(int k) { return k <= 12 ? 24 : (k <= 20 ? 32 : std::min(k + 12, kMaxK1v2)); }
+
 // Length of the register lists that serve lists of K1, 0 if they are too long.
 static int bf2_reg_list(int K1) { return K1 == 24 || K1 == 32 ? K1 : 0; }
 
@@ -1363,8 +1368,6 @@ static esg_status bf2_escalate(const PreparedX &X, const float *base, int64_t n,
     return st;
 }
 
-// One pass of the pipelined kernel over a batch of queries against the
-// prepared points, then merge, re-rank, certificate and escalation.
 // Cuts the sequence of covered point tiles (query tile by query tile) into G
 // contiguous shares of about equal estimated cost. A share's cost is its
 // number of tiles plus, for every row with a list, a weight for starting it: a
@@ -1686,35 +1689,57 @@ static esg_status bf2_plan(const int64_t *hl, const int64_t *hr, int64_t nq, int
     return ESG_OK;
 }
 
-// Writes out the covered tiles of the work items (a block each) from the query
-// tiles' spans. Inside an item the tiles are rotated to begin at the first one
-// at or after a multiple of `period`, about the length of the long items: the
-// CTAs that sweep the same points with different query tiles then read the same
-// blocks at about the same time, and the operand blocks come from DRAM once
-// instead of once per query tile (DRAM reads 10.7 -> 5.7 GB at 1M x
-// 128, 5.5 -> 2.2 GB at 200,003 x 768, whose call takes 1.54 ms instead of 1.65).
+// The covered tiles of a work item in the order its CTA takes them: rotated to
+// begin at the first one at or after a multiple of `period`, about the length
+// of the long items. The CTAs that sweep the same points with different query
+// tiles then read the same blocks at about the same time, and the operand blocks
+// come from DRAM once instead of once per query tile (DRAM reads 10.7 -> 5.7 GB
+// at 1M x 128, 5.5 -> 2.2 GB at 200,003 x 768, whose call takes 1.54 ms instead
+// of 1.65). The spans are the query tiles' (Spans).
+struct ItemTiles {
+    const int32_t *a;
+    const int64_t *at;
+    int32_t x0, x1, cnt, lead;
+    int64_t off;
+    __host__ __device__ ItemTiles(const WorkItem &w, const int32_t *span_a, const int32_t *span_first,
+                                  const int64_t *span_at, int period)
+        : a(span_a), at(span_at), x0(span_first[w.qtile]), x1(span_first[w.qtile + 1]), cnt(w.cnt), off(w.off) {
+        const int64_t from = ((int64_t)ascending(off) + period - 1) / period * period;
+        int lo = 0, hi = cnt;
+        while (lo < hi) {
+            const int m = (lo + hi) >> 1;
+            if (ascending(off + m) < from) lo = m + 1; else hi = m;
+        }
+        lead = lo;
+    }
+    __host__ __device__ int32_t ascending(int64_t pos) const {
+        int32_t x = x1 - 1;
+        while (x > x0 && at[x] > pos) --x;
+        return a[x] + (int32_t)(pos - at[x]);
+    }
+    __host__ __device__ int32_t operator[](int j) const {
+        return ascending(off + (lead + (int64_t)j < cnt ? lead + j : lead + j - cnt));
+    }
+};
+
+// The rotation's period: an upper quartile of the items' lengths.
+static int bf2_period(const std::vector<WorkItem> &items) {
+    std::vector<int32_t> c(items.size());
+    for (size_t i = 0; i < items.size(); ++i) c[i] = items[i].cnt;
+    std::nth_element(c.begin(), c.begin() + c.size() * 3 / 4, c.end());
+    return c[c.size() * 3 / 4];
+}
+
+// Writes out the covered tiles of the work items, a block each.
 __global__ void expand_tiles_kernel(const WorkItem *items, const int32_t *span_a, const int32_t *span_first,
                                     const int64_t *span_at, int period, int32_t *tiles) {
     const WorkItem w = items[blockIdx.x];
-    const int32_t x0 = span_first[w.qtile], x1 = span_first[w.qtile + 1];
-    auto tile = [&](int64_t pos) {
-        int32_t x = x1 - 1;
-        while (x > x0 && span_at[x] > pos) --x;
-        return span_a[x] + (int32_t)(pos - span_at[x]);
-    };
-    // the first tile of the item at or after a multiple of the period
-    const int32_t first = tile(w.off), from = (first + period - 1) / period * period;
-    int lo = 0, hi = w.cnt;
-    while (lo < hi) {
-        const int m = (lo + hi) >> 1;
-        if (tile(w.off + m) < from) lo = m + 1; else hi = m;
-    }
-    for (int j = threadIdx.x; j < w.cnt; j += blockDim.x) {
-        const int k = lo + j < w.cnt ? lo + j : lo + j - w.cnt;
-        tiles[w.off + j] = tile((int64_t)w.off + k);
-    }
+    const ItemTiles t(w, span_a, span_first, span_at, period);
+    for (int j = threadIdx.x; j < w.cnt; j += blockDim.x) tiles[w.off + j] = t[j];
 }
 
+// One pass of the pipelined kernel over a batch of queries against the
+// prepared points, then merge, re-rank, certificate and escalation.
 // `given`: a plan already made for these ranges (it is consumed), or null. Where
 // memory is too short for the dense rows' buffer the pass goes without it.
 static esg_status bf2_queries(const PreparedX &X, const float *base, int64_t n, int32_t d, int metric,
@@ -1805,12 +1830,8 @@ static esg_status bf2_queries(const PreparedX &X, const float *base, int64_t n, 
                                  cudaMemcpyHostToDevice, stream);
         if (ce == cudaSuccess) {
             esg_fault_host();
-            std::vector<int32_t> c(n_items);
-            for (int64_t i = 0; i < n_items; ++i) c[i] = items[i].cnt;
-            std::nth_element(c.begin(), c.begin() + n_items * 3 / 4, c.end());
-            const int period = c[n_items * 3 / 4];
             expand_tiles_kernel<<<(unsigned)n_items, 256, 0, stream>>>(d_items, d_span_a, d_span_first, d_span_at,
-                                                                       period, d_tiles);
+                                                                       bf2_period(items), d_tiles);
             ce = cudaGetLastError();
         }
     }
@@ -1904,11 +1925,8 @@ static esg_status bf2_queries(const PreparedX &X, const float *base, int64_t n, 
 static esg_status bruteforce_tc_v2(const float *base, int64_t n, int32_t d, int metric, const float *queries,
                                    int64_t nq, const int64_t *l, const int64_t *r, int32_t k, int64_t *out_ids,
                                    float *out_dist, int32_t *out_count, cudaStream_t stream) {
-    // k + 12 candidates (the register lists' 24 or 32 for k up to 20), at least
-    // k + 8 (the longest list the kernel holds caps it): at 1M x 128, 10k
-    // queries, k = 10, lists of k + 8 left 2 queries uncertified, k + 12 certified all
     if (k < 1 || k + 8 > kMaxK1v2 || n >= ((int64_t)1 << 31) || d < 1) return ESG_ERR_UNSUPPORTED;
-    const int K1 = k <= 12 ? 24 : (k <= 20 ? 32 : std::min(k + 12, kMaxK1v2));
+    const int K1 = bf2_list(k);
     int dev = 0, max_smem = 0, S = 0, n_acc = 0;
     bool stream_a = false, list_smem = false;
     size_t smem = 0;
@@ -1988,31 +2006,9 @@ esg_status esg_bruteforce_tc(const float *base, int64_t n, int32_t d, int metric
     return st;
 }
 
-esg_status esg_bruteforce_plan(int64_t n, int32_t d, const int64_t *l, const int64_t *r, int64_t nq,
-                               int32_t ctas, int64_t *sizes, int32_t *order, int32_t *tiles, int32_t *items,
-                               int32_t *cta_first) {
-    if (n < 1 || n >= ((int64_t)1 << 31) - 1 || d < 1 || nq < 0 || nq >= ((int64_t)1 << 31) || ctas < 1 ||
-        !sizes || (nq > 0 && (!l || !r))) {
-        esg_set_error("esg_bruteforce_plan: bad argument");
-        return ESG_ERR_INVALID_ARG;
-    }
-    Bf2Plan P;
-    esg_status st = ESG_OK;
-    try {
-        st = bf2_plan(l, r, nq, n, d, ctas, false, 0, P);
-    } catch (...) { st = ESG_ERR_OOM; }
-    if (st != ESG_OK) {
-        if (st == ESG_ERR_UNSUPPORTED) esg_set_error("esg_bruteforce_plan: more than 2^31 covered point tiles");
-        return st;
-    }
-    sizes[0] = P.nv;
-    sizes[1] = P.total_tiles;
-    sizes[2] = (int64_t)P.items.size();
-    sizes[3] = P.G;
+// The parts of a plan that both inspection calls return.
+static void copy_plan(const Bf2Plan &P, int32_t *order, int32_t *items, int32_t *cta_first) {
     if (order) std::copy(P.order.begin(), P.order.end(), order);
-    if (tiles)
-        for (size_t x = 0; x < P.spans.a.size(); ++x)
-            for (int32_t t = P.spans.a[x]; t <= P.spans.b[x]; ++t) *tiles++ = t;
     if (items)
         for (size_t i = 0; i < P.items.size(); ++i) {
             items[4 * i] = P.items[i].qtile;
@@ -2021,5 +2017,62 @@ esg_status esg_bruteforce_plan(int64_t n, int32_t d, const int64_t *l, const int
             items[4 * i + 3] = 0;
         }
     if (cta_first) std::copy(P.cta_first.begin(), P.cta_first.end(), cta_first);
+}
+
+static esg_status inspect_plan(const char *who, int64_t n, int32_t d, const int64_t *l, const int64_t *r, int64_t nq,
+                               int32_t ctas, const int64_t *sizes, bool run, int K1, Bf2Plan &P) {
+    if (n < 1 || n >= ((int64_t)1 << 31) - 1 || d < 1 || nq < 0 || nq >= ((int64_t)1 << 31) || ctas < 1 ||
+        !sizes || (nq > 0 && (!l || !r))) {
+        esg_set_error(std::string(who) + ": bad argument");
+        return ESG_ERR_INVALID_ARG;
+    }
+    esg_status st = ESG_OK;
+    try {
+        st = bf2_plan(l, r, nq, n, d, ctas, run, K1, P);
+    } catch (...) { st = ESG_ERR_OOM; }
+    if (st == ESG_ERR_UNSUPPORTED) esg_set_error(std::string(who) + ": more than 2^31 covered point tiles");
+    return st;
+}
+
+esg_status esg_bruteforce_plan(int64_t n, int32_t d, const int64_t *l, const int64_t *r, int64_t nq,
+                               int32_t ctas, int64_t *sizes, int32_t *order, int32_t *tiles, int32_t *items,
+                               int32_t *cta_first) {
+    Bf2Plan P;
+    const esg_status st = inspect_plan("esg_bruteforce_plan", n, d, l, r, nq, ctas, sizes, false, 0, P);
+    if (st != ESG_OK) return st;
+    sizes[0] = P.nv;
+    sizes[1] = P.total_tiles;
+    sizes[2] = (int64_t)P.items.size();
+    sizes[3] = P.G;
+    if (tiles)
+        for (size_t x = 0; x < P.spans.a.size(); ++x)
+            for (int32_t t = P.spans.a[x]; t <= P.spans.b[x]; ++t) *tiles++ = t;
+    copy_plan(P, order, items, cta_first);
+    return ESG_OK;
+}
+
+esg_status esg_bruteforce_search_plan(int64_t n, int32_t d, int32_t k, const int64_t *l, const int64_t *r, int64_t nq,
+                                      int32_t ctas, int64_t *sizes, int32_t *order, int32_t *tiles, int32_t *items,
+                                      int32_t *cta_first, int64_t *dense) {
+    if (k < 1 || k + 8 > kMaxK1v2) {
+        esg_set_error("esg_bruteforce_search_plan: k outside the tensor-core path");
+        return ESG_ERR_INVALID_ARG;
+    }
+    Bf2Plan P;
+    const esg_status st = inspect_plan("esg_bruteforce_search_plan", n, d, l, r, nq, ctas, sizes, true, bf2_list(k), P);
+    if (st != ESG_OK) return st;
+    sizes[0] = P.nv;
+    sizes[1] = P.total_tiles;
+    sizes[2] = (int64_t)P.items.size();
+    sizes[3] = P.G;
+    sizes[4] = P.dense;
+    sizes[5] = P.items.empty() ? 0 : bf2_period(P.items);
+    if (tiles)
+        for (const WorkItem &w : P.items) {
+            const ItemTiles t(w, P.spans.a.data(), P.spans.first.data(), P.spans.at.data(), (int)sizes[5]);
+            for (int j = 0; j < w.cnt; ++j) tiles[w.off + j] = t[j];
+        }
+    copy_plan(P, order, items, cta_first);
+    if (dense) std::copy(P.doff.begin(), P.doff.end(), dense);
     return ESG_OK;
 }
