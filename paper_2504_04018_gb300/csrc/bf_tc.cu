@@ -1377,12 +1377,20 @@ static esg_status bf2_escalate(const PreparedX &X, const float *base, int64_t n,
 // together and share that cost, rows whose ranges begin inside it hardly do;
 // a dense row costs a little for each of its tiles (its stores). The shares
 // are chosen greedily: each CTA takes about the remaining cost over the
-// remaining CTAs; a later pass (of the inspected plan) adds the restart cost of
+// remaining CTAs; a second pass, where the shares are uneven, adds the restart cost of
 // the previous pass's later cuts to the remaining cost, and the pass with the
 // smallest largest share is kept. `lt`/`rt` are the first and last covered
 // tile of each sorted query; `cut` receives G + 1 positions.
 constexpr double kRestart2 = 6.25;   // one list start, in tiles, at two K chunks
-constexpr int kSharePasses = 2;      // greedy passes (the first without restart look-ahead)
+// Greedy passes (the first without restart look-ahead), and the excess of the
+// largest share over the mean, in tiles at two K chunks, from which the second
+// one pays: it takes the host 25 to 100 us, a tile takes a CTA about 1.1 us.
+// Without it the largest share is 10 % above the mean at 1M x 128, 10k queries
+// and k = 10 but 43 % at k = 100, and 2.5 times the mean with 1,000 queries. A call
+// over 1M points takes 11.0 ms with it and 15.6 without (3,000 queries over all x
+// 96, k = 100), 0.91 and 1.08 ms (1,000 over 600,000 x 128, k = 10).
+constexpr int kSharePasses = 2;
+constexpr double kShareSlack = 32.0;
 
 // In tiles: a row whose range begins inside the item, one that begins before
 // it (its list starts with the item, along with the other rows' lists), and a
@@ -1404,7 +1412,7 @@ struct Spans {
 
 static void bf2_shares(const Spans &sp, const std::vector<int64_t> &qt_first, const std::vector<int32_t> &lt,
                        const std::vector<int32_t> &rt, const std::vector<int32_t> &dense, int64_t G,
-                       const ShareCost &w, int passes, std::vector<int64_t> &cut) {
+                       const ShareCost &w, double slack, std::vector<int64_t> &cut) {
     const int64_t nqt = (int64_t)qt_first.size() - 1, T = qt_first[nqt];
     const int64_t nv = (int64_t)lt.size();
     cut.assign(G + 1, T);
@@ -1493,7 +1501,8 @@ static void bf2_shares(const Spans &sp, const std::vector<int64_t> &qt_first, co
     std::vector<int64_t> cur, nxt;
     double best = greedy(later, cur);
     cut = cur;
-    for (int pass = 1; pass < passes; ++pass) {
+    const double mean = pre[nqt] / (double)G;
+    for (int pass = 1; pass < kSharePasses && best - mean > std::max(slack, 0.02 * mean); ++pass) {
         // restart cost of each cut of the previous pass (the next share's head
         // plus the query tile's cost up to the cut, minus the whole query
         // tile), summed over the later cuts
@@ -1656,7 +1665,7 @@ static esg_status bf2_plan(const int64_t *hl, const int64_t *hr, int64_t nq, int
         const double c = K1 > 32 ? K1 / 24.0 : 1.0;   // insertions grow with the list
         const ShareCost w = run ? ShareCost{16.0 * c * g, 0.5 * c * g, 0.0104 * g}
                                 : ShareCost{kRestart2 * f * f, kRestart2 * f * f, 0.0};
-        bf2_shares(sp, qt_first, lt, rt, dense, G, w, run ? 1 : kSharePasses, cut);
+        bf2_shares(sp, qt_first, lt, rt, dense, G, w, kShareSlack * f, cut);
     }
     std::vector<WorkItem> &items = P.items;
     items.clear();

@@ -1,6 +1,7 @@
 """The plan that a tensor-core exact search runs (esg_bruteforce_search_plan, no
 GPU work): its order and coverage are the inspected plan's, its dense rows fit
-their buffer, and a work item's tiles are a rotation."""
+their buffer, a work item's tiles are a rotation, and the shares balance the
+costs it is made by."""
 import numpy as np
 import pytest
 
@@ -9,6 +10,25 @@ import synthetic
 E = pytest.importorskip("paper_2504_04018_gb300")
 
 TM = TN = 128
+
+
+def _costs(d, k, l, r, order, tiles, items, cta_first, dense):
+    """Cost of each CTA's share by the header's formula."""
+    nk = -(-d // 64)
+    f = 2.0 / nk
+    g = f if nk <= 2 else f ** 3
+    c = min(k + 12, 128) / 24.0 if k > 20 else 1.0
+    lt, rt = l[order] // TN, r[order] // TN
+    cost = np.empty(len(items))
+    for i, (qt, off, cnt, _) in enumerate(items):
+        a, b = tiles[off:off + cnt].min(), tiles[off:off + cnt].max()
+        q = slice(qt * TM, min(len(order), (qt + 1) * TM))
+        lo, hi = np.maximum(lt[q], a), np.minimum(rt[q], b)
+        over, dn = lo <= hi, dense[q] >= 0
+        begin = over & (lt[q] > a) & ~dn
+        cost[i] = (cnt + 16.0 * c * g * begin.sum() + 0.5 * c * g * (over & ~dn & ~begin).sum() +
+                   0.0104 * g * (hi - lo + 1)[over & dn].sum())
+    return np.array([cost[cta_first[c]:cta_first[c + 1]].sum() for c in range(len(cta_first) - 1)])
 
 
 def check(n, d, k, l, r, ctas=152):
@@ -84,3 +104,14 @@ def test_search_plan_halves_the_dense_width(k, nq):
     l = (rng.random(nq) * (n - w)).astype(np.int64)
     dense = check(n, 96, k, l, l + w - 1)[4]
     assert (dense >= 0).any() and (dense < 0).any()
+
+
+def test_search_plan_balances_its_cost():
+    """Widths 2^-j N (j = 0..10) over 1M points: the largest share stays within
+    15 % of the mean, as in the inspected plan."""
+    n = 1_000_000
+    for nq, d, k in ((10_000, 128, 10), (10_000, 768, 10), (10_000, 96, 100), (1000, 128, 10)):
+        l, r = synthetic.ranges_from_fractions(n, 2.0 ** -(np.arange(nq) % 11).astype(np.float64), 77)
+        order, tiles, items, cta_first, dense, _, _ = check(n, d, k, l, r)
+        cost = _costs(d, k, l, r, order, tiles, items, cta_first, dense)
+        assert cost.max() <= 1.15 * cost.mean(), (nq, d, k, cost.max() / cost.mean())
