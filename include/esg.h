@@ -499,7 +499,16 @@ esg_status esg_query_budget(const esg_index *index, const float *queries, int64_
  *  k         1..1024;
  *  out_ids   device [nq, k] int64 row indices, out_dist device [nq, k] float32,
  *  out_count device [nq] int32.
- * Asynchronous on `stream`.
+ * Calls on the tensor cores (k up to 120) return when their results are ready:
+ * the host reads the ranges, plans, and reads the certificates. Their scratch is
+ * 256 bytes per point and 64 dimensions, up to 1 GiB (2 GiB past k = 20) for the
+ * distances of narrow ranges, and 16 bytes per list entry, two lists per query and
+ * work item; the library's pool keeps it for later calls (up to ESG_POOL_KEEP_MB,
+ * 8 GiB by default). Above k = 120, and with ceil(d / 64) = 1 and k > 56 or more
+ * dimensions and k > 50 for sets of a few hundred points or under stream capture,
+ * the call is asynchronous on `stream` and takes no scratch up to k = 128; with
+ * these k and few narrow ranges it waits only for the ranges. The answers are the
+ * same either way.
  */
 esg_status esg_bruteforce_filtered_knn(const float *base, int64_t n, int32_t d, esg_metric metric,
                                        const float *queries, int64_t nq, const int64_t *l,

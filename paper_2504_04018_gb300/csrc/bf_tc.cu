@@ -1251,6 +1251,84 @@ static bool bf2_serial(int32_t d, int k) { return k + 8 > ((d + TK - 1) / TK == 
 // 10k queries, k = 10, lists of k + 8 left 2 queries uncertified, k + 12 certified all.
 static int bf2_list(int k) { return k <= 12 ? 24 : (k <= 20 ? 32 : std::min(k + 12, kMaxK1v2)); }
 
+// Where both paths give the same answers (bf2_serial), the one that takes less
+// time by these estimates serves the call: a few narrow ranges are a few point
+// tiles of the SIMT kernel, while the tensor-core path prepares all points and
+// makes a host plan first. In us, fitted to 682 pairs of timed calls (1 to 4,096
+// queries, 1,000 to 10M points, 32 to 768 dimensions, ranges of 100 points to all,
+// k = 60 and 100): of those where the two are over 15 % apart, all take the faster.
+// One query over 1,000 of 1M x 96 points, k = 100: 281 us on the tensor cores, 232
+// us in the SIMT kernel with the look at the ranges; over 1,000 of 10M x 96: 1,552
+// and 232; over 10,000 of 1M x 96: 297 and 1,550; 4,096 over all of 1,000 x 256:
+// 2,529 and 840.
+// The SIMT kernel: a CTA per 64 queries, two of them on an SM, takes the 64-point
+// tiles one of its queries covers, passes over the others between them, and a
+// warp folds a tile into its eight queries' lists one after the other.
+constexpr double kLook = 22.0;   // reading the ranges first
+struct SimtCost {
+    double tile, fold;
+    int64_t slots;
+    SimtCost(int32_t d, int k, int64_t sms) : tile(3.0 + 0.06 * d), fold(1.3 + 0.02 * k), slots(2 * sms) {}
+    // a CTA whose queries lie in a hull of `hull` tiles and cover `sum` of them,
+    // `fold_tiles` the eight of one warp (at most)
+    double cta(int64_t hull, int64_t sum, int64_t fold_tiles) const {
+        return 0.18 * hull + tile * std::min(sum, hull) + fold * fold_tiles;
+    }
+};
+
+// All queries over all points: what any ranges take at most.
+static double simt_us_at_most(int64_t n, int64_t nq, int32_t d, int k, int64_t sms) {
+    const SimtCost c(d, k, sms);
+    const int64_t t = (n + 63) / 64, ctas = (nq + 63) / 64;
+    return 30.0 + c.cta(t, t, t * std::min<int64_t>(nq, 8)) * std::max(1.0, (double)ctas / c.slots);
+}
+
+static double simt_us(const std::vector<int64_t> &l, const std::vector<int64_t> &r, int64_t n, int32_t d, int k,
+                      int64_t sms) {
+    const SimtCost c(d, k, sms);
+    const int64_t nq = (int64_t)l.size();
+    double most = 0.0, all = 0.0;
+    for (int64_t q0 = 0; q0 < nq; q0 += 64) {
+        int64_t lo = n, hi = -1, sum = 0, fold = 0;
+        for (int64_t w = q0; w < std::min(nq, q0 + 64); w += 8) {
+            int64_t warp = 0;
+            for (int64_t q = w; q < std::min(nq, w + 8); ++q) {
+                if (l[q] < 0 || l[q] > r[q] || r[q] >= n) continue;
+                lo = std::min(lo, l[q]);
+                hi = std::max(hi, r[q]);
+                warp += (r[q] - l[q]) / 64 + 1;
+            }
+            sum += warp;
+            fold = std::max(fold, warp);
+        }
+        if (hi < 0) continue;
+        const double t = c.cta((hi - lo) / 64 + 1, sum, fold);
+        most = std::max(most, t);
+        all += t;
+    }
+    return 30.0 + std::max(most, all / c.slots);
+}
+
+// The tensor-core path: launches, host round trips and the plan; the points'
+// preparation (memory bound); and, past 128 dimensions, where narrow ranges keep
+// lists too, the insertions while these fill: a warp's rows, as far as their ranges
+// (`mean` points wide) lie in the item's tiles, one after the other. Wide ranges
+// take more than this, and the SIMT kernel much more.
+static double tc_us(int64_t n, int64_t nq, int64_t mean, int32_t d, int k, int64_t sms) {
+    const int64_t nk = (d + TK - 1) / TK;
+    double t = 140.0 + 0.05 * d + n * (4.0 * d + (double)STAGE / TM * nk) / 6.6e6;
+    if (nk > 2 && mean > 0) {
+        const double qt = std::ceil(nq / (double)TM), tiles = std::ceil(n / (double)TN);
+        const double ctas = std::min<double>(sms, qt * tiles), items = std::max(1.0, ctas / qt);
+        const double m = std::min<double>(n / items, mean) / 2, K1 = k + 12;   // points a list sees
+        const double ins = m <= K1 ? m : K1 * (1.0 + std::log(m / K1));
+        const double share = std::min(1.0, (mean + TN) / (n * std::min(1.0, TM / (double)nq) + mean));
+        t += 0.25 * (1.0 + (nk - 4) / 16.0) * ins * std::ceil(std::min<double>(nq, TM) / 4) *
+             std::max(1.0, qt * items / ctas) * share;
+    }
+    return t;
+}
+
 // Length of the register lists that serve lists of K1, 0 if they are too long.
 static int bf2_reg_list(int K1) { return K1 == 24 || K1 == 32 ? K1 : 0; }
 
@@ -1954,6 +2032,12 @@ static esg_status bruteforce_tc_v2(const float *base, int64_t n, int32_t d, int 
     ESG_CUDA_TRY(cudaMemcpyAsync(hl.data(), l, sizeof(int64_t) * nq, cudaMemcpyDeviceToHost, stream));
     ESG_CUDA_TRY(cudaMemcpyAsync(hr.data(), r, sizeof(int64_t) * nq, cudaMemcpyDeviceToHost, stream));
     ESG_CUDA_TRY(cudaStreamSynchronize(stream));
+    if (bf2_serial(d, k)) {
+        int64_t sum = 0;
+        for (int64_t i = 0; i < nq; ++i)
+            if (hl[i] >= 0 && hl[i] <= hr[i] && hr[i] < n) sum += hr[i] - hl[i] + 1;
+        if (kLook + simt_us(hl, hr, n, d, k, sms) < tc_us(n, nq, sum / nq, d, k, sms)) return ESG_ERR_UNSUPPORTED;
+    }
     auto al = [](size_t x) { return (x + 255) & ~(size_t)255; };
     const size_t bytes = al((size_t)xt * nk * STAGE) + al(sizeof(float) * xt * TN) + al(sizeof(float) * 4);
     Scratch scratch(stream);
@@ -1989,9 +2073,10 @@ static esg_status bruteforce_tc_v2(const float *base, int64_t n, int32_t d, int 
 
 // Tensor-core path of esg_bruteforce_filtered_knn; returns ESG_ERR_UNSUPPORTED
 // when the shape is outside it (the caller then uses the SIMT kernel). Where the
-// SIMT kernel gives the same answers bit for bit (bf2_serial), it also serves
-// calls that this path cannot: it needs no scratch memory and no host
-// synchronisation, so it runs when memory is short and under stream capture.
+// SIMT kernel gives the same answers bit for bit (bf2_serial), it also serves the
+// calls it answers sooner and those that this path cannot: it needs no scratch
+// memory and no host synchronisation, so it runs when memory is short and under
+// stream capture.
 esg_status esg_bruteforce_tc(const float *base, int64_t n, int32_t d, int metric, const float *queries,
                              int64_t nq, const int64_t *l, const int64_t *r, int32_t k, int64_t *out_ids,
                              float *out_dist, int32_t *out_count, cudaStream_t stream) {
@@ -2000,6 +2085,11 @@ esg_status esg_bruteforce_tc(const float *base, int64_t n, int32_t d, int metric
         cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
         if (cudaStreamIsCapturing(stream, &cs) != cudaSuccess) cudaGetLastError();
         if (cs != cudaStreamCaptureStatusNone) return ESG_ERR_UNSUPPORTED;
+        // small enough whatever the ranges are: no look at them, no host synchronisation
+        int dev = 0, sms = 0;
+        ESG_CUDA_TRY(cudaGetDevice(&dev));
+        ESG_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+        if (simt_us_at_most(n, nq, d, k, sms) < tc_us(n, nq, 0, d, k, sms)) return ESG_ERR_UNSUPPORTED;
     }
     esg_status st;
     try {

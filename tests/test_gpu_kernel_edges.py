@@ -307,3 +307,28 @@ def test_exact_host_failure_gives_scratch_back():
     out = subprocess.run([sys.executable, "-c", _HOST_FAILURE], env=env, capture_output=True, text=True, timeout=300,
                          cwd=os.path.dirname(os.path.dirname(os.path.abspath(__file__))))
     assert out.returncode == 0 and out.stdout.strip().endswith("ok"), out.stderr[-2000:]
+
+
+@pytest.mark.parametrize("n,nq,w,tensor", [(1_000_000, 1, 1000, False), (1_000_000, 1, 100_000, True),
+                                           (1_000_000, 64, 1000, True), (700, 1, 700, False), (60, 500, 60, False),
+                                           (2_000_000, 3, 100, False)])
+@pytest.mark.parametrize("k", [57, 100])
+def test_exact_long_lists_take_the_shorter_path(n, nq, w, tensor, k, monkeypatch):
+    """A few narrow ranges, and small sets, are answered by the SIMT kernel without
+    preparing the points; the answers do not depend on the path."""
+    g = torch.Generator(device=DEV).manual_seed(n + nq)
+    X = torch.randn(n, 32, generator=g, device=DEV)
+    Q = torch.randn(nq, 32, generator=g, device=DEV)
+    l = np.random.default_rng(n).integers(n // 2, n // 2 + 200 + 1, nq) if n > 1000 else np.zeros(nq, np.int64)
+    r = l + w - 1
+    E.esg_profile_enable(True)
+    try:
+        a = E.esg_bruteforce_filtered_knn(X, Q, _t(l), _t(r), k)
+        torch.cuda.synchronize()
+        assert (E.esg_profile_tensor_work() > 0) == tensor
+    finally:
+        E.esg_profile_enable(False)
+    monkeypatch.setenv("ESG_BF_SIMT", "1")
+    b = E.esg_bruteforce_filtered_knn(X, Q, _t(l), _t(r), k)
+    torch.cuda.synchronize()
+    assert all(torch.equal(x, y) for x, y in zip(a, b))
