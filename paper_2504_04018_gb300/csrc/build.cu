@@ -28,6 +28,7 @@
 #include "decompose.cuh"
 
 #include <algorithm>
+#include <cstdlib>
 #include <vector>
 
 #include <cub/cub.cuh>
@@ -81,10 +82,11 @@ __device__ __forceinline__ void row_dists(const float *xa, const float *const (&
 // later ones left are taken at once, the warps sharing them four at a time,
 // instead of one candidate after the other against the kept ones (the same
 // decisions). As many of the pool's rows as fit are staged in shared memory:
-// every step reads them. Latency bound: max_keep steps of about 1,000 cycles.
-// The forward edges of a 10,000 x 128 build (M = 16, pools of 200) took 19.2 ms
-// with a warp per point and one distance at a time, 7.2 ms now; the re-selected
-// rows 11.7 ms and 3.1 ms.
+// every step reads them. Latency bound: max_keep steps of about 1,000 cycles, and
+// about twice the distances that occlusion_select_warp takes, with two points on
+// an SM: for rounds that do not fill the device (kWarpRound). The forward edges
+// of a 10,000 x 128 build (M = 16, pools of 200) take 7.1 ms, 12.0 ms by warps;
+// the re-selected rows 2.8 and 6.6 ms.
 __device__ int occlusion_select(const float *X, int d, int metric, const Cand *pool, int m, int max_keep,
                                 uint32_t *keep, uint32_t *alive, float *stage) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -135,6 +137,44 @@ __device__ int occlusion_select(const float *X, int d, int metric, const Cand *p
     return kept;
 }
 
+// The same by a warp: one candidate after the other against the kept ones, which
+// takes no distance too many. Throughput bound in the large rounds of a large
+// build, where thousands of warps run: the forward edges of a 1M x 96 build (M = 32)
+// take 378 ms, 1,106 ms by blocks, and its re-selected rows 38 and 46 ms; 1M x 128
+// (M = 16) 273 and 960 ms, 81 and 202 ms.
+__device__ int occlusion_select_warp(const float *X, int d, int metric, const Cand *pool, int m, int max_keep,
+                                     uint32_t *keep) {
+    int kept = 0;
+    for (int i = 0; i < m && kept < max_keep; ++i) {
+        const uint32_t c = pool[i].id & ESG_ID_MASK;
+        const float *xc = X + (size_t)c * d;
+        const float dcb = pool[i].d;
+        bool good = true;
+        for (int s = 0; s < kept; ++s) {
+            const float *xs[1] = {X + (size_t)keep[s] * d};
+            float dist[1];
+            row_dists<1>(xc, xs, d, metric, dist);
+            if (dist[0] < dcb) { good = false; break; }
+        }
+        if (good) {
+            if ((threadIdx.x & 31) == 0) keep[kept] = c;
+            __syncwarp();
+            ++kept;
+        }
+    }
+    return kept;
+}
+
+// Points of a round from which its forward edges go by warps (in proportion past
+// 384 dimensions, where a block's rows do not fit its shared memory either), and
+// rows to re-select, in resident blocks, above which these do. Blocks win at 1,024
+// points x 128 (0.18 against 0.26 ms) and 512 to 768 x 768 (0.21 and 0.52), warps
+// at 2,048 to 3,955 x 96 (18.0 and 13.1 ms) and 4,096 to 7,910 x 768 (121 and 88).
+// A block re-selects a row about 8 times as fast as a warp: the lines cross at
+// 2,326 to 4,092 rows x 96 (5.6 ms each).
+constexpr int64_t kWarpRound = 2048;
+constexpr int kWarpRows = 8;
+
 // Block sort of P (a power of two) candidates in shared memory, ascending.
 __device__ void block_sort(Cand *v, int P) {
     for (int size = 2; size <= P; size <<= 1)
@@ -163,6 +203,24 @@ __global__ void __launch_bounds__(kEdgeThreads) forward_kernel(const float *X, i
     uint32_t *row = adj_depth + p * (int64_t)R;
     for (int j = threadIdx.x; j < R; j += kEdgeThreads) {
         const uint32_t v = j < kept ? keep[j] : ESG_NONE;
+        row[j] = v;
+        if (v != ESG_NONE) atomicAdd(&indeg[v], 1);
+    }
+}
+
+// The same, a warp per point.
+__global__ void __launch_bounds__(128) forward_warp_kernel(const float *X, int d, int metric, int64_t n_items,
+                                                           const int64_t *pts, const Cand *res, const int32_t *res_cnt,
+                                                           int efc, int M, int R, uint32_t *adj_depth, int32_t *indeg) {
+    __shared__ uint32_t keep_s[4][kMaxRow];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int64_t it = blockIdx.x * (int64_t)4 + w;
+    if (it >= n_items) return;
+    const int64_t p = pts[it];
+    const int kept = occlusion_select_warp(X, d, metric, res + it * (int64_t)efc, res_cnt[it], M, keep_s[w]);
+    uint32_t *row = adj_depth + p * (int64_t)R;
+    for (int j = lane; j < R; j += 32) {
+        const uint32_t v = j < kept ? keep_s[w][j] : ESG_NONE;
         row[j] = v;
         if (v != ESG_NONE) atomicAdd(&indeg[v], 1);
     }
@@ -206,17 +264,18 @@ __global__ void reverse_append_kernel(int64_t n, int R, const int64_t *off, cons
     }
 }
 
-// The listed points' rows, a block each: re-selected by occlusion among the (at
-// most kMaxPool) closest of old row + new sources.
+// The listed points' rows, a block each, if there are at most `most`: re-selected
+// by occlusion among the (at most kMaxPool) closest of old row + new sources.
 __global__ void __launch_bounds__(kEdgeThreads) reselect_kernel(const float *X, int d, int metric, int R,
                                                                 const int64_t *off, const int32_t *indeg,
                                                                 const uint32_t *rev, const int32_t *full,
-                                                                const int32_t *n_full, uint32_t *adj_depth) {
+                                                                const int32_t *n_full, int most, uint32_t *adj_depth) {
     extern __shared__ __align__(16) float stage[];
     __shared__ Cand pool[2 * kMaxPool];
     __shared__ uint32_t keep[kMaxRow], alive[1024 / 32];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int count = *n_full;
+    if (count > most) return;
     for (int f = blockIdx.x; f < count; f += gridDim.x) {
         const int64_t v = full[f];
         const int nr = indeg[v];
@@ -257,6 +316,57 @@ __global__ void __launch_bounds__(kEdgeThreads) reselect_kernel(const float *X, 
     }
 }
 
+// The same, a warp each, if there are more.
+__global__ void __launch_bounds__(128) reselect_warp_kernel(const float *X, int d, int metric, int R, const int64_t *off,
+                                                            const int32_t *indeg, const uint32_t *rev,
+                                                            const int32_t *full, const int32_t *n_full, int most,
+                                                            uint32_t *adj_depth) {
+    __shared__ Cand pool_s[4][2 * kMaxPool];
+    __shared__ uint32_t keep_s[4][kMaxRow];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    Cand *pool = pool_s[w];
+    const int count = *n_full;
+    if (count <= most) return;
+    for (int f = blockIdx.x * 4 + w; f < count; f += gridDim.x * 4) {
+        const int64_t v = full[f];
+        const int nr = indeg[v];
+        uint32_t *row = adj_depth + v * (int64_t)R;
+        const uint32_t *src = rev + off[v];
+        int deg = 0;   // rows are packed left
+        for (int b0 = 0; b0 < R; b0 += 32)
+            deg += __popc(__ballot_sync(0xffffffffu, b0 + lane < R && row[b0 + lane] != ESG_NONE));
+        const int total = deg + nr;
+        const float *xv = X + (size_t)v * d;
+        int m = 0;
+        // kMaxPool candidates at a time beside the kMaxPool closest so far
+        for (int c0 = 0; c0 < total; c0 += kMaxPool) {
+            const int nc = min(kMaxPool, total - c0);
+            for (int g = 0; g < nc; g += 4) {
+                uint32_t id[4];
+                const float *xb[4];
+                float dist[4];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const int j = min(c0 + g + k, total - 1);
+                    id[k] = j < deg ? row[j] : src[j - deg];
+                    xb[k] = X + (size_t)id[k] * d;
+                }
+                row_dists<4>(xv, xb, d, metric, dist);
+                if (lane == 0)
+                    for (int k = 0; k < 4 && g + k < nc; ++k) pool[m + g + k] = Cand{dist[k], id[k]};
+            }
+            const int mm = m + nc, P = next_pow2_int(max(mm, 2));
+            for (int t = mm + lane; t < P; t += 32) pool[t] = Cand{INFINITY, ESG_NONE};
+            __syncwarp();
+            warp_sort_pow2(pool, P);
+            m = min(mm, kMaxPool);
+        }
+        const int kept = occlusion_select_warp(X, d, metric, pool, m, R, keep_s[w]);
+        for (int j = lane; j < R; j += 32) row[j] = j < kept ? keep_s[w][j] : ESG_NONE;
+        __syncwarp();
+    }
+}
+
 struct HostNode { int64_t l, r; int32_t heap; };
 
 // Graph nodes (r - l >= leaf) at `depth` of the fanout-f tree over [0, n-1].
@@ -289,6 +399,8 @@ struct Rounds {
     size_t cub_bytes = 0;
     int64_t cap = 0;
     int blocks = 0;   // resident blocks of the edge kernels
+    int64_t warp_round = 0;   // rounds of this many points go by warps
+    int warp_rows = 0;        // as do more rows than this to re-select
     ~Rounds() {
         cudaFree(pts); cudaFree(pieces); cudaFree(res); cudaFree(res_cnt); cudaFree(stats);
         cudaFree(indeg); cudaFree(cursor); cudaFree(full); cudaFree(off); cudaFree(rev); cudaFree(bentry);
@@ -313,6 +425,9 @@ esg_status rounds_alloc(Rounds &B, const esg_index *ix, int64_t cap, int efc, in
     int sms = 0;
     B_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ix->device));
     B.blocks = 2 * sms;
+    const char *wr = getenv("ESG_BUILD_WARP_ROUND");
+    B.warp_round = wr && *wr ? std::max(1ll, atoll(wr)) : kWarpRound * std::max(384, ix->d) / 384;
+    B.warp_rows = wr && *wr ? (int)std::min<int64_t>(B.warp_round - 1, INT32_MAX) : kWarpRows * B.blocks;
     B_TRY(cudaFuncSetAttribute(forward_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kStageBytes));
     B_TRY(cudaFuncSetAttribute(reselect_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kStageBytes));
     B_TRY(esg_malloc((void **)&B.rev, sizeof(uint32_t) * cap * M));
@@ -342,16 +457,29 @@ esg_status insert_round(esg_index *ix, const esg_build_params &p, Rounds &B, int
     if (st != ESG_OK) return st;
     B_TRY(cudaMemsetAsync(B.cursor, 0, sizeof(int32_t) * n, stream));
     B_TRY(cudaMemsetAsync(B.full, 0, sizeof(int32_t), stream));
-    forward_kernel<<<(unsigned)ni, kEdgeThreads, kStageBytes, stream>>>(ix->X, d, ix->metric, B.pts, B.res, B.res_cnt,
-                                                                        efc, M, R, adj_t, B.indeg);
+    const bool warps = ni >= B.warp_round;
+    if (warps)
+        forward_warp_kernel<<<ceil_div_i(ni, 4), 128, 0, stream>>>(ix->X, d, ix->metric, ni, B.pts, B.res, B.res_cnt,
+                                                                   efc, M, R, adj_t, B.indeg);
+    else
+        forward_kernel<<<(unsigned)ni, kEdgeThreads, kStageBytes, stream>>>(ix->X, d, ix->metric, B.pts, B.res,
+                                                                            B.res_cnt, efc, M, R, adj_t, B.indeg);
     B_TRY(cudaGetLastError());
     B_TRY(cub::DeviceScan::ExclusiveSum(B.cub_tmp, B.cub_bytes, B.indeg, B.off, (int)(n + 1), stream));
     scatter_reverse_kernel<<<ceil_div_i(ni, 256), 256, 0, stream>>>(ni, B.pts, M, R, adj_t, B.off, B.cursor, B.rev);
     B_TRY(cudaGetLastError());
     reverse_append_kernel<<<ceil_div_i(n, 4), 128, 0, stream>>>(n, R, B.off, B.indeg, B.rev, adj_t, B.full + 1, B.full);
-    reselect_kernel<<<B.blocks, kEdgeThreads, kStageBytes, stream>>>(ix->X, d, ix->metric, R, B.off, B.indeg, B.rev,
-                                                                     B.full + 1, B.full, adj_t);
     B_TRY(cudaGetLastError());
+    // how many rows are listed only the device knows: of two kernels one returns
+    reselect_kernel<<<B.blocks, kEdgeThreads, kStageBytes, stream>>>(ix->X, d, ix->metric, R, B.off, B.indeg, B.rev,
+                                                                     B.full + 1, B.full, warps ? B.warp_rows : INT32_MAX,
+                                                                     adj_t);
+    B_TRY(cudaGetLastError());
+    if (warps) {
+        reselect_warp_kernel<<<B.blocks * 4, 128, 0, stream>>>(ix->X, d, ix->metric, R, B.off, B.indeg, B.rev,
+                                                               B.full + 1, B.full, B.warp_rows, adj_t);
+        B_TRY(cudaGetLastError());
+    }
     B_TRY(cudaMemsetAsync(B.indeg, 0, sizeof(int32_t) * (n + 1), stream));
     B_TRY(cudaStreamSynchronize(stream));
     return ESG_OK;

@@ -332,3 +332,23 @@ def test_exact_long_lists_take_the_shorter_path(n, nq, w, tensor, k, monkeypatch
     b = E.esg_bruteforce_filtered_knn(X, Q, _t(l), _t(r), k)
     torch.cuda.synchronize()
     assert all(torch.equal(x, y) for x, y in zip(a, b))
+
+
+@pytest.mark.parametrize("d,M,efc,n", [(32, 4, 40, 6000), (128, 16, 200, 5000), (768, 8, 100, 3000)])
+@pytest.mark.parametrize("metric", ["l2", "ip"])
+def test_build_by_warps_is_the_build_by_blocks(d, M, efc, n, metric, monkeypatch):
+    """Rounds of one to half of the points, every round's edges by blocks, by warps,
+    and by the rule's choice: the same rows (as sets)."""
+    rng = np.random.default_rng(d)
+    X = rng.standard_normal((n, d)).astype(np.float32)
+    rows = []
+    for points in (str(1 << 30), "1", None):
+        if points is None:
+            monkeypatch.delenv("ESG_BUILD_WARP_ROUND")
+        else:
+            monkeypatch.setenv("ESG_BUILD_WARP_ROUND", points)
+        ix = E.esg_build(X, None, M=M, leaf_size=64, n_entries=8, ef_construction=efc, batch_div=1, metric=metric)
+        adj, _, _ = E.esg_index_export(ix)
+        assert np.all(np.diff((adj == 0xFFFFFFFF).astype(np.int8), axis=-1) >= 0)
+        rows.append(np.sort(adj, axis=-1))
+    assert np.array_equal(rows[0], rows[1]) and np.array_equal(rows[0], rows[2])
