@@ -352,3 +352,15 @@ def test_build_by_warps_is_the_build_by_blocks(d, M, efc, n, metric, monkeypatch
         assert np.all(np.diff((adj == 0xFFFFFFFF).astype(np.int8), axis=-1) >= 0)
         rows.append(np.sort(adj, axis=-1))
     assert np.array_equal(rows[0], rows[1]) and np.array_equal(rows[0], rows[2])
+
+
+@pytest.mark.parametrize("B", [9727, 9728, 9729, 30_001])
+def test_mlp_forward_block_edges(B):
+    """Chunks of 8 rows on at most 1,216 blocks: blocks with one and several."""
+    rng = np.random.default_rng(B)
+    F = E.esg_mlp_num_features()
+    p = (rng.standard_normal(OM.n_params(F)) * 0.2).astype(np.float32)
+    X = (rng.standard_normal((B, F)) * 2 + 0.5).astype(np.float32)
+    mu, sigma = rng.standard_normal(F).astype(np.float32), (rng.random(F) + 0.5).astype(np.float32)
+    y = E.esg_mlp_forward(_t(p), _t(X), _t(mu), _t(sigma)).cpu().numpy()
+    assert np.allclose(y, OM.forward(p, X, mu, sigma)[0], rtol=1e-5, atol=1e-5)
