@@ -3,6 +3,7 @@
 #include "esg_internal.cuh"
 
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
@@ -110,12 +111,15 @@ struct FaultCounter {
     std::mutex mu;
     std::string seen;
     long long count = 0;
+    std::atomic<bool> on{false};   // a value is set: the next call without one resets
     explicit FaultCounter(const char *n) : name(n) {}
     bool hit() {
         const char *v = getenv(name);
+        if ((!v || !*v) && !on.load(std::memory_order_relaxed)) return false;
         const std::string cur = v ? v : "";
         std::lock_guard<std::mutex> lk(mu);
         if (cur != seen) { seen = cur; count = 0; }   // a new value starts a new count
+        on.store(!cur.empty(), std::memory_order_relaxed);
         if (cur.empty()) return false;
         const long long k = atoll(cur.c_str());
         return k >= 1 && ++count == k;

@@ -1455,20 +1455,22 @@ static esg_status bf2_escalate(const PreparedX &X, const float *base, int64_t n,
 // together and share that cost, rows whose ranges begin inside it hardly do;
 // a dense row costs a little for each of its tiles (its stores). The shares
 // are chosen greedily: each CTA takes about the remaining cost over the
-// remaining CTAs; a second pass, where the shares are uneven, adds the restart cost of
+// remaining CTAs; a second pass, where the shares are uneven (always in the
+// inspected plan of plain lists), adds the restart cost of
 // the previous pass's later cuts to the remaining cost, and the pass with the
 // smallest largest share is kept. `lt`/`rt` are the first and last covered
 // tile of each sorted query; `cut` receives G + 1 positions.
 constexpr double kRestart2 = 6.25;   // one list start, in tiles, at two K chunks
 // Greedy passes (the first without restart look-ahead), and the excess of the
-// largest share over the mean, in tiles at two K chunks, from which the second
-// one pays: it takes the host 25 to 100 us, a tile takes a CTA about 1.1 us.
-// Without it the largest share is 10 % above the mean at 1M x 128, 10k queries
-// and k = 10 but 43 % at k = 100, and 2.5 times the mean with 1,000 queries. A call
-// over 1M points takes 11.0 ms with it and 15.6 without (3,000 queries over all x
-// 96, k = 100), 0.91 and 1.08 ms (1,000 over 600,000 x 128, k = 10).
+// largest share over the mean from which the second one pays, as a part of the
+// mean and in tiles at two K chunks: it takes the host 25 to 100 us, a tile takes
+// a CTA about 1.1 us. Without it the largest share is 10 % above the mean at 1M x
+// 128, 10k queries and k = 10, where a call takes 2.79 ms without it and 2.84 with
+// it, but 43 % at k = 100, and 2.5 times the mean with 1,000 queries: 11.0 ms with
+// it and 15.6 without (3,000 queries over all of 1M x 96, k = 100), 0.91 and 1.08
+// ms (1,000 over 600,000 of 1M x 128, k = 10).
 constexpr int kSharePasses = 2;
-constexpr double kShareSlack = 32.0;
+constexpr double kShareUneven = 0.15, kShareSlack = 32.0;
 
 // In tiles: a row whose range begins inside the item, one that begins before
 // it (its list starts with the item, along with the other rows' lists), and a
@@ -1490,7 +1492,7 @@ struct Spans {
 
 static void bf2_shares(const Spans &sp, const std::vector<int64_t> &qt_first, const std::vector<int32_t> &lt,
                        const std::vector<int32_t> &rt, const std::vector<int32_t> &dense, int64_t G,
-                       const ShareCost &w, double slack, std::vector<int64_t> &cut) {
+                       const ShareCost &w, double uneven, double slack, std::vector<int64_t> &cut) {
     const int64_t nqt = (int64_t)qt_first.size() - 1, T = qt_first[nqt];
     const int64_t nv = (int64_t)lt.size();
     cut.assign(G + 1, T);
@@ -1580,7 +1582,7 @@ static void bf2_shares(const Spans &sp, const std::vector<int64_t> &qt_first, co
     double best = greedy(later, cur);
     cut = cur;
     const double mean = pre[nqt] / (double)G;
-    for (int pass = 1; pass < kSharePasses && best - mean > std::max(slack, 0.02 * mean); ++pass) {
+    for (int pass = 1; pass < kSharePasses && best - mean >= std::max(slack, uneven * mean); ++pass) {
         // restart cost of each cut of the previous pass (the next share's head
         // plus the query tile's cost up to the cut, minus the whole query
         // tile), summed over the later cuts
@@ -1743,7 +1745,7 @@ static esg_status bf2_plan(const int64_t *hl, const int64_t *hr, int64_t nq, int
         const double c = K1 > 32 ? K1 / 24.0 : 1.0;   // insertions grow with the list
         const ShareCost w = run ? ShareCost{16.0 * c * g, 0.5 * c * g, 0.0104 * g}
                                 : ShareCost{kRestart2 * f * f, kRestart2 * f * f, 0.0};
-        bf2_shares(sp, qt_first, lt, rt, dense, G, w, kShareSlack * f, cut);
+        bf2_shares(sp, qt_first, lt, rt, dense, G, w, run ? kShareUneven : 0.0, run ? kShareSlack * f : 0.0, cut);
     }
     std::vector<WorkItem> &items = P.items;
     items.clear();
@@ -1791,7 +1793,7 @@ struct ItemTiles {
     __host__ __device__ ItemTiles(const WorkItem &w, const int32_t *span_a, const int32_t *span_first,
                                   const int64_t *span_at, int period)
         : a(span_a), at(span_at), x0(span_first[w.qtile]), x1(span_first[w.qtile + 1]), cnt(w.cnt), off(w.off) {
-        const int64_t from = ((int64_t)ascending(off) + period - 1) / period * period;
+        const int32_t from = (ascending(off) + period - 1) / period * period;   // tiles below 2^24
         int lo = 0, hi = cnt;
         while (lo < hi) {
             const int m = (lo + hi) >> 1;
@@ -1805,7 +1807,8 @@ struct ItemTiles {
         return a[x] + (int32_t)(pos - at[x]);
     }
     __host__ __device__ int32_t operator[](int j) const {
-        return ascending(off + (lead + (int64_t)j < cnt ? lead + j : lead + j - cnt));
+        const uint32_t i = (uint32_t)lead + (uint32_t)j;
+        return ascending(off + (i < (uint32_t)cnt ? i : i - (uint32_t)cnt));
     }
 };
 
