@@ -6,8 +6,8 @@
 // and the split residuals are below 2^-17 relative). Queries are sorted and
 // tiled by 128 (one TMEM lane each); a query tile visits the 128-point tiles
 // its ranges cover (128 TMEM columns per tile). The pipelined kernel below
-// is warp-specialised: bulk copies of pre-swizzled operand blocks, one MMA
-// thread, and eight epilogue warps that keep the K1 best approximate
+// is warp-specialised: bulk copies of pre-swizzled operand blocks, two MMA
+// threads, and eight epilogue warps that keep the K1 best approximate
 // distances per query.
 //
 // A second kernel merges a query's lists, recomputes exact FP32 distances
@@ -216,13 +216,13 @@ __device__ __forceinline__ void sort_asc(Key (&L)[NL], int lane) {
 //               commits them to mbarriers;
 //   warps 3..10 epilogue, two groups of four warps (one per TMEM lane
 //               quarter) that take alternate tiles. A thread owns one query
-//               row: it reads the row's 128 columns 8 or 16 at a time, compares
+//               row: it reads the row's 128 columns 32 at a time, compares
 //               each distance with the row's threshold and appends the few
 //               that pass to the row's pending slots in shared memory. When a
-//               row's slots run low its warp sorts them in registers and
-//               merges them into the row's sorted list in global memory (32
-//               NL keys across the lanes, the loads overlapped with the
-//               sort), which lowers the threshold. At d <= 256 group 0 also
+//               row's slots run low all rows of the warp insert theirs into
+//               lists of 24 or 32 held in registers, or (longer lists) the
+//               warp merges the rows' by ranks into their lists in global
+//               memory, which lowers the threshold. At d <= 256 group 0 also
 //               puts the item's query tile into tensor memory (64 columns per
 //               64 dimensions): the MMAs then read only the point operand from
 //               shared memory, which at N = 128 otherwise limits them, and
@@ -255,11 +255,11 @@ constexpr int kMaxK1v2 = 128;             // longest list
 constexpr int kMaxStages = 6;
 constexpr int kTmem = 512;                // TMEM columns: all, one CTA per SM
 constexpr int kMaxResident = 4;           // 64-wide chunks of a query tile that fit beside two accumulators
-// Columns between two checks of the pending slots, slots per row (a check's
-// columns must fit, at most 32: one per lane of the sort), and how many of
-// them make a row worth merging along with one that has to be. 20 slots leave
-// room for four stages and the lists at d = 128, K1 = 22; 12 for three streamed
-// stages.
+// Columns between two checks of the pending slots, slots per row where the lists
+// are in memory (a check's columns must fit, at most 32: one per lane of the
+// merge), and how many of them make a row worth merging along with one that has
+// to be. 20 slots leave room for five stages, 12 for three streamed stages. Rows
+// with register lists have 16 (kPend in the kernel): five stages, two streamed.
 constexpr int kCols = 8;
 template <bool STREAM> struct Epi {
     static constexpr int kPend = STREAM ? 12 : 20, kFill = STREAM ? 4 : 8;
@@ -286,7 +286,7 @@ struct Tc2Args {
     int n_items;
     int64_t nv;                     // number of valid (sorted) queries
     int nk, metric, K1, S;
-    int list_smem;                  // 1: lists in shared memory while they grow
+    int list_smem;                  // 1: lists of up to 64 in shared memory while they grow
     int n_acc;                      // TMEM accumulators
     int issuers;                    // MMA-issuing threads, 1 or 2
     int64_t n;                      // points
@@ -478,6 +478,7 @@ __global__ void __launch_bounds__(kThreads2, 1) tc_knn2_kernel(Tc2Args a) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     constexpr int kPend = KR ? 16 : Epi<STREAM>::kPend, kFill = Epi<STREAM>::kFill;
     constexpr int kStride = KR ? 32 : kPendStride;   // lists in registers: a slot's 32 rows side by side
+    constexpr bool kSmemLists = KR == 0 && NL <= 2;   // see bf2_smem
     const int K1 = a.K1;
     // tile n of the CTA's run uses accumulator n mod n_acc and barrier n mod
     // n_bar, an even number: all uses of a barrier belong to one issuer and
@@ -691,7 +692,7 @@ __global__ void __launch_bounds__(kThreads2, 1) tc_knn2_kernel(Tc2Args a) {
                 }
             }
             Key *out = a.part + (((int64_t)it * 2 + group) * TM + quarter * 32) * K1;
-            Key *list = a.list_smem ? s_list + ew * 32 * K1 : out;
+            Key *list = kSmemLists && a.list_smem ? s_list + ew * 32 * K1 : out;
             const int64_t sp = (int64_t)I.qtile * TM + my_row;
             int32_t lo = 1, hi = 0;
             float *drow = nullptr;   // a dense row's distance of point p goes to drow[p]
@@ -848,7 +849,7 @@ __global__ void __launch_bounds__(kThreads2, 1) tc_knn2_kernel(Tc2Args a) {
                         st.len = e + 1;
                     }
                 }
-            } else if (a.list_smem) {
+            } else if (kSmemLists && a.list_smem) {
                 for (int r = 0; r < 32; ++r) {
                     const int m = __shfl_sync(0xffffffffu, st.len, r);
 #pragma unroll
@@ -1349,10 +1350,14 @@ static esg_status bf2_smem(int32_t d, int K1, int max_smem, int *S, size_t *smem
     size_t common = sizeof(float2) * kEpiWarps * pend * (reg ? 32 : kPendStride) + sizeof(float) * kEpiWarps * TN +
                     sizeof(Key) * 4 * TM + 8 * (2 * kMaxStages + 16) + 16;
     if ((size_t)max_smem < common + 2 * stage) return ESG_ERR_UNSUPPORTED;
-    // the lists in shared memory where they leave four stages (a list in
-    // global memory is a trip to the L2, busy with operand blocks, per merge)
+    // the lists in shared memory where they leave four stages (a list in global
+    // memory is a trip to the L2, busy with operand blocks, per merge). With 227
+    // KB none of K1 > 32 do: 33 at d <= 256 need 249 KB. The kernel of lists up to
+    // 64 keeps the choice because without it the compiler's code for it is slower
+    // (398 queries over 219,744 x 256, k = 50: 676 -> 688 us a call); that of longer
+    // lists is faster (10k over 1M x 96, k = 100: 9.29 -> 8.60 ms).
     const size_t lists = sizeof(Key) * 2 * TM * K1;
-    *list_smem = !reg && (size_t)max_smem >= common + lists + 4 * stage;
+    *list_smem = !reg && K1 <= 64 && (size_t)max_smem >= common + lists + 4 * stage;
     if (*list_smem) common += lists;
     *S = (int)std::min<size_t>(kMaxStages, ((size_t)max_smem - common) / stage);
     *smem = common + (size_t)*S * stage;
@@ -1630,7 +1635,7 @@ struct Bf2Plan {
 // are dense, in a buffer twice as large (1M x 96, 10k queries, k = 100: 9.5 ms a
 // call, 179 ms through the SIMT kernel).
 constexpr int64_t kDenseWidth = 131072;
-constexpr int64_t kDenseFloats = (int64_t)1 << 28;   // 1 GiB at most
+constexpr int64_t kDenseFloats = (int64_t)1 << 28;   // 1 GiB at most (2 GiB with lists in memory)
 
 static void bf2_dense(const int64_t *hl, const int64_t *hr, int64_t widest, int64_t most, Bf2Plan &P) {
     P.doff.assign(P.order.size(), -1);
@@ -1715,7 +1720,7 @@ static esg_status bf2_plan(const int64_t *hl, const int64_t *hr, int64_t nq, int
     // the rows of each full query tile interleaved over the four TMEM lane
     // quarters (sorted position s -> row (s mod 4) * 32 + s / 4): queries
     // with nearby ranges take their insertions in the same point tiles, and
-    // an accumulator is free only when all four epilogue warp pairs are done
+    // an accumulator is free only when all four warps of its group are done
     for (int64_t qt = 0; qt < nv / TM; ++qt) {
         int32_t rows[TM];
         for (int i = 0; i < TM; ++i) rows[(i & 3) * 32 + (i >> 2)] = order[qt * TM + i];
@@ -1933,7 +1938,7 @@ static esg_status bf2_queries(const PreparedX &X, const float *base, int64_t n, 
         if (nqt > 0)
             ce = split_norm(queries, nv, d, nk, d_order, nqt * TM, qs, qnorm, qrow, nullptr, stream);
     }
-    // lists in 32 or 64 registers-times-lanes
+    // lists of 24 or 32 in registers, or in memory: 64 or 128 keys over a warp's lanes
     const bool l2 = metric == ESG_L2SQ, one = K1 <= 32, two = K1 <= 64;
     auto pick = [&](auto s) -> void (*)(Tc2Args) {
         constexpr bool ST = decltype(s)::value;
