@@ -71,7 +71,7 @@ __device__ __forceinline__ void row_dists(const float *xa, const float *const (&
 #pragma unroll
     for (int w = 0; w < W; ++w) {
         const float r = warp_sum_group(acc[w], 32);
-        out[w] = metric == ESG_L2SQ ? r : -r;
+        out[w] = ordered_dist(metric == ESG_L2SQ ? r : -r);
     }
 }
 

@@ -223,6 +223,11 @@ struct Cand {
     uint32_t id;  // bit 31: expanded flag (search lists only)
 };
 
+// A computed distance as lists take it: NaN (a NaN element, or inner products of
+// infinite terms) counts as +inf. Sorts and merges place every candidate only if
+// the distances are ordered; an unplaced one would leave an undefined id in a list.
+__device__ __forceinline__ float ordered_dist(float d) { return fminf(d, INFINITY); }
+
 __device__ __forceinline__ bool cand_less(float da, uint32_t ia, float db, uint32_t ib) {
     return da < db || (da == db && (ia & ESG_ID_MASK) < (ib & ESG_ID_MASK));
 }

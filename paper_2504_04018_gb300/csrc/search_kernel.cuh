@@ -379,7 +379,7 @@ __device__ __forceinline__ void eval_rows(const uint4 *__restrict__ Xv, const fl
                 acc = accum_vec<ST>(xv[u][v], qs + (s + v * LPR) * EPV, sc[u], metric, acc);
             acc = warp_sum_group(acc, LPR);
             const int row = base + u * rows_per_pass + g;
-            if (s == 0 && row < m) batch[row] = Cand{metric == ESG_L2SQ ? acc : -acc, id[u]};
+            if (s == 0 && row < m) batch[row] = Cand{ordered_dist(metric == ESG_L2SQ ? acc : -acc), id[u]};
         }
     }
     __syncwarp();
@@ -412,7 +412,7 @@ __device__ __forceinline__ void eval_rows_fp32(const float *__restrict__ X, int 
             }
         }
         acc = warp_sum_group(acc, 8);
-        if (s == 0 && row < m) out[row] = Cand{metric == ESG_L2SQ ? acc : -acc, id};
+        if (s == 0 && row < m) out[row] = Cand{ordered_dist(metric == ESG_L2SQ ? acc : -acc), id};
     }
     __syncwarp();
 }

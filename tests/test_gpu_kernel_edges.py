@@ -364,3 +364,42 @@ def test_mlp_forward_block_edges(B):
     mu, sigma = rng.standard_normal(F).astype(np.float32), (rng.random(F) + 0.5).astype(np.float32)
     y = E.esg_mlp_forward(_t(p), _t(X), _t(mu), _t(sigma)).cpu().numpy()
     assert np.allclose(y, OM.forward(p, X, mu, sigma)[0], rtol=1e-5, atol=1e-5)
+
+
+@pytest.mark.parametrize("metric", ["l2", "ip"])
+@pytest.mark.parametrize("rows", ["f32", "bf16", "fp8"])
+def test_search_orders_nan_distances(metric, rows):
+    """NaN elements in points and queries, and inner products of infinite terms:
+    such points are at +inf, each point comes at most once and from its range,
+    and queries without them are answered as without them."""
+    n, d, k, nq = 3000, 32, 20, 64
+    rng = np.random.default_rng(7)
+    X = rng.standard_normal((n, d)).astype(np.float32)
+    bad = rng.choice(n, 90, replace=False)
+    X[bad[:30], 0] = np.nan
+    X[bad[30:60]] = np.nan
+    X[bad[60:]] = np.where(np.arange(d) % 2, np.float32(3e37), np.float32(-3e37))
+    q = rng.standard_normal((nq, d)).astype(np.float32)
+    q[::4, 1] = np.nan
+    q[1::8] *= 100
+    w = np.where(np.arange(nq) % 2, 40, 2500)   # scanned leaf pieces and graph pieces
+    l = (rng.random(nq) * (n - w + 1)).astype(np.int64)
+    ix = E.esg_build(X, None, M=16, leaf_size=64, n_entries=16, ef_construction=100, metric=metric, storage=rows)
+    ids, dist, count, _ = (t.cpu().numpy() for t in E.esg_search_batch(
+        ix, _t(q), _t(l), _t(l + w - 1), None, k, params=E.search_params(256, traversal=rows))[:4])
+    is_bad = np.zeros(n, bool)
+    is_bad[bad] = True
+    for i in range(nq):
+        got, dd = ids[i, :count[i]], dist[i, :count[i]]
+        assert len(set(got.tolist())) == len(got) and np.all((got >= l[i]) & (got < l[i] + w[i]))
+        assert not np.isnan(dd).any() and np.all(dd[:-1] <= dd[1:])
+        if i % 4 == 0:
+            assert np.all(dd == np.inf)
+            continue
+        good = np.flatnonzero(~is_bad[l[i]:l[i] + w[i]]) + l[i]
+        got = got[dd < np.inf]
+        assert len(got) == k and (metric == "ip" or not is_bad[got].any())
+        if metric == "l2":
+            d64 = ((X[good].astype(np.float64) - q[i]) ** 2).sum(1)
+            want = good[np.argsort(d64)[:k]]
+            assert len(set(want.tolist()) & set(got.tolist())) >= 0.9 * k
