@@ -253,8 +253,10 @@ esg_status make_plan(int d, int R, int efk, int64_t n_items, int st, int width, 
         ESG_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm96, f96, pl.wpb * 32, pl.smem));
     }
     // automatic: the 96-register build only where more searches reside with
-    // it (at 10^7 points, d = 96, 100k queries: BF16 rows at ef 128 118.9
-    // vs 129.5 ms per call, FP8 116.5 vs 128.4)
+    // it. At 10^7 points, d = 96, 100k queries, ef 128, 96 against 128
+    // registers: two candidates expanded at a time 67.9 and 70.2 ms per call
+    // on BF16 rows, 67.1 and 71.4 on FP8; one at a time 73.3 and 71.4 on
+    // BF16 (44 bytes spilled), 71.0 and 71.6 on FP8. The autotuner times both.
     const bool use96 = mr_req == 96 || (mr_req == 0 && f96 != nullptr && per_sm96 > per_sm128);
     SearchFn fn = use96 ? f96 : f128;
     per_sm = use96 ? per_sm96 : per_sm128;

@@ -5,7 +5,7 @@
 namespace esg_sk {
 
 SearchFn pick_fp8(int vpl, bool occ5) {
-    if (occ5) {   // 96 registers, at most a few words spilled, for these splits
+    if (occ5) {   // 96 registers: 8 bytes spilled with one vector per lane, none with 3
         if (vpl == 1) return search_kernel<ESG_FP8E4M3, 1, 5>;
         if (vpl == 3) return search_kernel<ESG_FP8E4M3, 3, 5>;
         return nullptr;

@@ -619,7 +619,7 @@ struct SearchArgs {
 
 // MINB: resident blocks of 128 threads per SM the register allocation is
 // sized for (4: up to 128 registers; 5: up to 96, instantiated only where
-// that compiles with at most a few words spilled).
+// that compiles with at most 44 bytes spilled).
 template <int ST, int VPL, int MINB = 4>
 __global__ void __launch_bounds__(128, MINB)
 search_kernel(SearchArgs a) {
