@@ -309,7 +309,8 @@ esg_status esg_decompose_batch(int64_t n, int32_t leaf_size, esg_layout layout, 
  *  k           device [nq] int32 per-query k (1..k_max), or NULL for k_max;
  *  k_max       1..1024, row stride of the outputs;
  *  out_ids     device [nq, k_max] int64: original ids (via the re-ranking);
- *  out_dist    device [nq, k_max] float32 distances;
+ *  out_dist    device [nq, k_max] float32 distances, ascending; NaN counts as
+ *              +inf;
  *  out_count   device [nq] int32: results written, min(k, r - l + 1) when the
  *              graphs reach enough in-range points;
  *  out_status  device [nq] int32 (ESG_Q_* bits) or NULL;
