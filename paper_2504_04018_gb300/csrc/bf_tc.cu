@@ -238,7 +238,9 @@ __device__ __forceinline__ void sort_asc(Key (&L)[NL], int lane) {
 // 0.74 us, and the CTAs take 1.1 to 1.2 us per tile: an accumulator is held for
 // the MMAs and then for the group's reading, three of them are in turn, and
 // everything that passes the shared-memory crossbar (norms, shuffles, pending
-// slots) competes with the MMAs' operand reads. 4.67 -> 2.0 ms for the kernel,
+// slots) competes with the MMAs' operand reads. The operand blocks come from
+// DRAM at 79 % of the copy bandwidth meanwhile (10.0 GB read, 0.85 GB written in
+// 2.05 ms), the tensor pipe is active in half of the cycles. 4.67 -> 2.0 ms for the kernel,
 // 1.52 -> 1.07 ms at 200,003 x 768 (2k queries), 256 -> 18 us for 61 queries over
 // 99,991 x 100. Tried on the way: one issuer (a thread's waits and commits cost
 // as much as a stage's MMAs), lists sorted by shuffle networks of 4 or 8 rows
@@ -1786,10 +1788,10 @@ static esg_status bf2_plan(const int64_t *hl, const int64_t *hr, int64_t nq, int
 // The covered tiles of a work item in the order its CTA takes them: rotated to
 // begin at the first one at or after a multiple of `period`, about the length
 // of the long items. The CTAs that sweep the same points with different query
-// tiles then read the same blocks at about the same time, and the operand blocks
-// come from DRAM once instead of once per query tile (DRAM reads 10.7 -> 5.7 GB
-// at 1M x 128, 5.5 -> 2.2 GB at 200,003 x 768, whose call takes 1.54 ms instead
-// of 1.65). The spans are the query tiles' (Spans).
+// tiles then read the same blocks at about the same time, more of them from the
+// L2 (without and with it, DRAM reads and the kernel: 10,000 queries over 1M x 128
+// 11.8 and 10.0 GB, 2.15 and 2.05 ms; 2,000 over 200,000 x 768 5.4 and 1.8 GB,
+// 1.18 and 1.07 ms). The spans are the query tiles' (Spans).
 struct ItemTiles {
     const int32_t *a;
     const int64_t *at;
